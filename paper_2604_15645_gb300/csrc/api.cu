@@ -150,6 +150,8 @@ pinn_status plan_call(const pinn_handle* h, int64_t n_res, int64_t n_ic, int64_t
       lp.nsplit = tc_adjdw_splits(h, lp.fin, c->p.NC);   // one partial per fused-kernel CTA and m-tile
     } else if (c->tc[li]) {
       lp.nsplit = tc_dw_splits(h, lp.fout, lp.fin, c->p.NC);
+    } else if (h->spec.precision != PINN_BF16) {
+      lp.nsplit = f32_dw_splits(lp.fout, lp.fin, c->p.NC, std::max(h->sm_count, 1));
     } else {
       const int tiles = ((lp.fout + 63) / 64) * ((lp.fin + 63) / 64);
       int ns = (4 * std::max(h->sm_count, 1) + tiles - 1) / tiles;
@@ -231,6 +233,7 @@ struct Pass {
 
   int nterms() const { return d_grad_terms ? 3 : 1; }
   const float* W32(int li) const { return reinterpret_cast<const float*>(ws + cp.lay[li].w32); }
+  const float* WT32(int li) const { return reinterpret_cast<const float*>(ws + cp.lay[li].wt32); }
   const float* bias(int li) const { return d_params + cp.lay[li].off_b; }
 
   pinn_status init(size_t ws_bytes) {
@@ -301,7 +304,8 @@ struct Pass {
     if (cp.tc[li])
       return tc_gemm_fwd(h, ws + cp.lay[li].wc, ws + cp.lay[li].wlo, ws + p.A[li], ws + p.Alo[li], cp.lay[li].fout,
                          cp.lay[li].fin, p.NC, e, st);
-    launch_simt_gemm_fwd(W32(li), ws + p.A[li], cp.lay[li].fout, cp.lay[li].fin, p.NP, e, prec, st);
+    launch_simt_gemm_fwd(W32(li), WT32(li), ws + p.A[li], cp.lay[li].fout, cp.lay[li].fin, p.NP, e, prec, h->sm_count,
+                         st);
     return PINN_OK;
   }
 
@@ -407,8 +411,8 @@ struct Pass {
                        st);
         if (s) return s;
       } else {
-        launch_simt_gemm_dw(zb, false, ws + p.A[li], false, lp.fout, lp.fin, p.NC, lp.nsplit,
-                            reinterpret_cast<float*>(ws + lp.dwpart), prec, st);
+        launch_simt_gemm_dw(zb, ws + p.A[li], lp.fout, lp.fin, p.NC, lp.nsplit, reinterpret_cast<float*>(ws + lp.dwpart),
+                            prec, st);
       }
     }
     if (!cp.fused_db[li] && !(li == L - 1 && cp.out_db)) {
@@ -421,8 +425,7 @@ struct Pass {
       // its contraction with the embedding's derivatives by B (or the periods).
       PhaseScope ps(h, st, PH_OTHER, 3);
       double* ffpart = reinterpret_cast<double*>(ws + p.ffpart);
-      launch_simt_gemm_lin(reinterpret_cast<const float*>(ws + lp.wt32), zb, lp.fin, lp.fout, p.NP, ws + p.Zbar[0],
-                           prec, st);
+      launch_simt_gemm_lin(WT32(li), W32(li), zb, lp.fin, lp.fout, p.NP, ws + p.Zbar[0], prec, h->sm_count, st);
       launch_ff_grad(ws + p.Zbar[0], b->x_res, b->x_ic, b->x_bc, p.n_res, p.n_ic, p.n_bc, h->d_in, h->ff_B,
                      h->spec.ff_m, mode, p.NP, ffpart, prec, st);
       launch_ff_grad_final(ffpart, h->d_in, h->spec.ff_m, h->periodic, h->periods, pc.first ? 0 : 1, d_grad_ff, st);
@@ -451,7 +454,7 @@ struct Pass {
       return tc_gemm_adj(h, ws + lp.wtc, ws + lp.wtlo, ws + cp.zbpm[(li + 1) % 2], lp.fin, lp.fout, p.NC, e, st);
     }
     if (cp.tc[li]) return tc_gemm_adj(h, ws + lp.wtc, nullptr, zb, lp.fin, lp.fout, p.NC, e, st);
-    launch_simt_gemm_adj(reinterpret_cast<const float*>(ws + lp.wt32), zb, lp.fin, lp.fout, p.NP, e, prec, st);
+    launch_simt_gemm_adj(WT32(li), W32(li), zb, lp.fin, lp.fout, p.NP, e, prec, h->sm_count, st);
     return PINN_OK;
   }
 

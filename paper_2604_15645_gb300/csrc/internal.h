@@ -166,19 +166,23 @@ struct EpiArgs {
   int64_t n_res, n_ic, n_bc;
 };
 
-// D[M][4 NP] = Aop[M][K] Bop[K][4 NP] (+ epilogue), Aop row-major ld=K (FP32 weights),
-// Bop row-major (activations in the compute type).
-void launch_simt_gemm_fwd(const float* Aop, const void* Bop, int M, int K, int64_t NP, const EpiArgs& e, int prec,
-                          cudaStream_t st);
-void launch_simt_gemm_adj(const float* Aop, const void* Bop, int M, int K, int64_t NP, const EpiArgs& e, int prec,
-                          cudaStream_t st);
-// out[M][4 NP] = Aop[M][K] Bop[K][4 NP] with no epilogue (the input-jet adjoint W_1^T Zbar_1).
-void launch_simt_gemm_lin(const float* Aop, const void* Bop, int M, int K, int64_t NP, void* out, int prec,
-                          cudaStream_t st);
-// part[s][M][N] = sum_{k in split s} Aop[m][k] Bop[n][k]; Aop/Bop row-major with ld = NC.
-// a_fp32 / b_fp32 select float storage, else the compute type.
-void launch_simt_gemm_dw(const void* Aop, bool a_fp32, const void* Bop, bool b_fp32, int M, int N, int64_t NC,
-                         int nsplit, float* part, int prec, cudaStream_t st);
+// CUDA-core GEMMs: D[M][4 NP] = A[M][K] Bop[K][4 NP] (+ epilogue), Bop the jets in the
+// compute type.  The FP32 weights are given in both orientations, [fout][fin] (W) and
+// [fin][fout] (WT); sms is the device's SM count.
+//   forward  A = W   (M = fout, K = fin)
+//   adjoint  A = W^T (M = fin, K = fout)
+//   lin      A = W^T with no epilogue (the input-jet adjoint W_1^T Zbar_1)
+void launch_simt_gemm_fwd(const float* W, const float* WT, const void* Bop, int M, int K, int64_t NP, const EpiArgs& e,
+                          int prec, int sms, cudaStream_t st);
+void launch_simt_gemm_adj(const float* WT, const float* W, const void* Bop, int M, int K, int64_t NP, const EpiArgs& e,
+                          int prec, int sms, cudaStream_t st);
+void launch_simt_gemm_lin(const float* WT, const float* W, const void* Bop, int M, int K, int64_t NP, void* out,
+                          int prec, int sms, cudaStream_t st);
+// part[s][M][N] = sum_{k in split s} Aop[m][k] Bop[n][k], both in the compute type, tile-major.
+void launch_simt_gemm_dw(const void* Aop, const void* Bop, int M, int N, int64_t NC, int nsplit, float* part, int prec,
+                         cudaStream_t st);
+// Column splits of the FP32 weight gradient.
+int f32_dw_splits(int M, int N, int64_t NC, int sms);
 
 struct OutArgs {
   const void* AL;        // A_L^T [w][NC] compute type

@@ -1,0 +1,34 @@
+"""Kernels at the sizes where their tiling can go wrong (tile edges, remainders, the
+smallest and largest of a dispatch rule's range), against the FP64 oracle at the
+precision's stated tolerance."""
+import numpy as np
+import pytest
+import torch
+
+from synth import NetSpec, Problem, ff_matrix, init_params, make_batch
+from synth.workloads import PDE_BURGERS, PDE_MAXWELL, PDE_NS
+
+from gpu_helpers import TOL, assert_parity, run_gpu, run_oracle
+
+pytestmark = pytest.mark.gpu
+
+
+def _parity(spec, n_res, n_ic, n_bc, precision, what):
+    p = init_params(spec, 71, 0.2)
+    B = ff_matrix(spec, 72)
+    b = make_batch(spec.pde, n_res, n_ic, n_bc, 73, 74)
+    prob = Problem(0.02, 0.3, 2.0, 5.0)
+    gt, gg = run_gpu(spec, p, B, b, prob, precision)
+    rt, rg = run_oracle(spec, p, B, b, prob, chunk=4096)
+    assert_parity(gt, gg, rt, rg, TOL[precision], what, spec=spec)
+
+
+@pytest.mark.parametrize("widths,ff,n_res", [
+    ([1, 3], 0, 1),                # a single point; 4-byte weight copies; one K step, mostly padding
+    ([66, 130, 17], 5, 95),        # widths past a 64- and a 128-feature block, M not a multiple of 4
+    ([64, 128, 64], 8, 4096),      # full blocks, 64-feature blocks at this size
+    ([80, 72], 24, 9800),          # the smallest sizes that take 128-feature blocks
+])
+def test_fp32_gemm_edges(cuda_lib, widths, ff, n_res):
+    spec = NetSpec(PDE_NS, 2, 3, widths, ff_m=ff, ff_sigma=1.0, rwf=True)
+    _parity(spec, n_res, 0, 33, "fp32", f"fp32 {widths} {n_res}")
