@@ -159,6 +159,32 @@ __device__ __forceinline__ void store_pm8(float* pm, int64_t c0, int M, int m, c
     for (int i = 0; i < 8; ++i) pm[(c0 + 64 * r + i) * M + m] = v[r][i];
 }
 
+// Coordinate terms of a raw first layer's weight gradient, dW_ij = sum_points zbar x_j +
+// sum over rows of direction j of zbar_j, in the adjoint epilogues.  Each warp covers 32
+// points of a tile for its 32 features: lane i looks up point i's coordinates once per tile
+// and the lanes exchange them by shuffles.  (Looking every point up in every lane
+// took 0.56 ms more of Maxwell 5x512's four adjoint launches, 3.57 -> 3.01 ms, and 11% of a
+// step of 64 networks.)
+__device__ __forceinline__ void lane_coords(const EpiArgs& e, int64_t point, float x[3]) {
+#pragma unroll
+  for (int j = 0; j < 3; ++j)
+    if (j < e.dterms) x[j] = point_coord(e.x_res, e.x_ic, e.x_bc, e.n_res, e.n_ic, e.n_bc, point, j);
+}
+template <int N>
+__device__ __forceinline__ void coord_terms(const float (&v)[4][N], const float x[3], int first, int dterms, int mode,
+                                            float db[4]) {
+  const int nd = (mode == JET_MAXWELL) ? 3 : 2;   // rows 1..nd are first derivatives
+#pragma unroll
+  for (int j = 0; j < 3; ++j)
+    if (j < dterms) {
+#pragma unroll
+      for (int i = 0; i < N; ++i) {
+        db[1 + j] = fmaf(v[0][i], __shfl_sync(0xffffffffu, x[j], first + i), db[1 + j]);
+        if (j < nd) db[1 + j] += v[1 + j][i];
+      }
+    }
+}
+
 // ---- the kernel -----------------------------------------------------------------------
 // SINE (BF16 forward / adjoint): the periodic activation sin(w0 z) instead of tanh.  Its
 // adjoint cannot be written in the activations (the sign of cos is lost), so the
@@ -447,6 +473,9 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA, const CUte
       const bool mvalid = m < p.M;
       const uint32_t tbase = tmem_base + ((uint32_t)(quad * 32) << 16) + (DW2 ? half : buf) * BN;
       float db[4] = {0.f, 0.f, 0.f, 0.f};
+      float xc[3] = {0.f, 0.f, 0.f};
+      if (MODE == TC_ADJ && p.e.dbpart && p.e.dterms)
+        lane_coords(p.e, (int64_t)nb * TILE_PTS + part * (UNITS * UPTS) + lane, xc);
 
       auto issue = [&](int u, float (&v)[4][UPTS]) {
 #pragma unroll
@@ -455,17 +484,8 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA, const CUte
           else tmem_ld16_issue(tbase + unit_col(u) + 64 * r, v[r]);
         }
       };
-      auto process = [&](int u, float (&v)[4][UPTS]) {
-        uint32_t zw[ZR][ZW];
-        if constexpr (MODE == TC_ADJ && !SINE) {
-#pragma unroll
-          for (int r = 0; r < ZR; ++r)
-#pragma unroll
-            for (int j = 0; j < ZW; ++j) zw[r][j] = znext[r][j];
-          if (u + 1 < UNITS) load_z(t, u + 1);
-          else if (t + grid.gdim() < total) load_z(t + grid.gdim(), 0);
-        }
-        if (!mvalid) return;
+      // the epilogue of one unit of a valid row
+      auto finish = [&](int u, float (&v)[4][UPTS], const uint32_t (&zw)[ZR][ZW]) {
         const int pc = unit_col(u);                                   // first point of the unit in its tile
         const int64_t cbase = toff(m, (int64_t)nb * BN, p.M) + pc;    // tile nb, row m
         if constexpr (MODE == TC_FWD) {
@@ -537,27 +557,6 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA, const CUte
           if constexpr (TF32) {
             if (p.e.out_pm) store_pm8(reinterpret_cast<float*>(p.e.out_pm), (int64_t)nb * BN + pc, p.M, m, v);
           }
-          if (p.e.dbpart) {
-            // bias gradient of the layer below (value rows) and, for a first layer on
-            // raw coordinates, the coordinate terms of its weight gradient
-#pragma unroll
-            for (int i = 0; i < UPTS; ++i) db[0] += v[0][i];
-            if (p.e.dterms) {
-              const int64_t p0 = (int64_t)nb * TILE_PTS + pc;
-              const int nd = (p.e.jet_mode == JET_MAXWELL) ? 3 : 2;   // rows 1..nd are first derivatives
-#pragma unroll
-              for (int i = 0; i < UPTS; ++i) {
-                const int64_t pp = p0 + i;
-#pragma unroll
-                for (int j = 0; j < 3; ++j) {
-                  if (j >= p.e.dterms) break;
-                  float x = point_coord(p.e.x_res, p.e.x_ic, p.e.x_bc, p.e.n_res, p.e.n_ic, p.e.n_bc, pp, j);
-                  db[1 + j] = fmaf(v[0][i], x, db[1 + j]);
-                  if (j < nd) db[1 + j] += v[1 + j][i];
-                }
-              }
-            }
-          }
         } else if constexpr (MODE == TC_DW) {
           const int split = t / (p.m_tiles * p.n_tiles);
           float* dst = p.out32 + ((int64_t)split * p.M + m) * p.N;
@@ -574,6 +573,26 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA, const CUte
         } else {   // TC_STORE
 #pragma unroll
           for (int r = 0; r < 4; ++r) st_f32<UPTS>(p.out32 + cbase + 64 * r, v[r]);
+        }
+      };
+      auto process = [&](int u, float (&v)[4][UPTS]) {
+        uint32_t zw[ZR][ZW];
+        if constexpr (MODE == TC_ADJ && !SINE) {
+#pragma unroll
+          for (int r = 0; r < ZR; ++r)
+#pragma unroll
+            for (int j = 0; j < ZW; ++j) zw[r][j] = znext[r][j];
+          if (u + 1 < UNITS) load_z(t, u + 1);
+          else if (t + grid.gdim() < total) load_z(t + grid.gdim(), 0);
+        }
+        if (mvalid) finish(u, v, zw);
+        if (MODE == TC_ADJ && p.e.dbpart) {
+          // bias gradient of the layer below (value rows) and, for a first layer on raw
+          // coordinates, the coordinate terms of its weight gradient (every lane: rows past M
+          // add values that nobody stores)
+#pragma unroll
+          for (int i = 0; i < UPTS; ++i) db[0] += v[0][i];
+          if (p.e.dterms) coord_terms<UPTS>(v, xc, UPTS * u, p.e.dterms, p.e.jet_mode, db);
         }
       };
 
@@ -1138,6 +1157,8 @@ __device__ __forceinline__ void tc_adjdw_body(const CUtensorMap* mapW, const CUt
       int mb, nb;
       coords(t, mb, nb);
       mb_cta = mb;
+      float xc[3] = {0.f, 0.f, 0.f};
+      if (p.e.dbpart && p.e.dterms) lane_coords(p.e, (int64_t)nb * TILE_PTS + part * 32 + lane, xc);
       if (!mbar_wait(acc_full, (uint32_t)local & 1, abort_flag, p.status, p.wait_ns)) break;
       tc_fence_after();
       float v[UNITS][4][UPTS];
@@ -1187,25 +1208,11 @@ __device__ __forceinline__ void tc_adjdw_body(const CUtensorMap* mapW, const CUt
           T* zbo = reinterpret_cast<T*>(p.e.out) + cbase;
 #pragma unroll
           for (int r = 0; r < 4; ++r) st_row(zbo + 64 * r, v[u][r]);
-          if (p.e.dbpart) {
+        }
+        if (p.e.dbpart) {   // (every lane: rows past M add zeros that nobody stores)
 #pragma unroll
-            for (int i = 0; i < UPTS; ++i) db[0] += v[u][0][i];
-            if (p.e.dterms) {
-              const int64_t p0 = (int64_t)nb * TILE_PTS + pc;
-              const int nd = (p.e.jet_mode == JET_MAXWELL) ? 3 : 2;
-#pragma unroll
-              for (int i = 0; i < UPTS; ++i) {
-                const int64_t pp = p0 + i;
-#pragma unroll
-                for (int j = 0; j < 3; ++j) {
-                  if (j >= p.e.dterms) break;
-                  float x = point_coord(p.e.x_res, p.e.x_ic, p.e.x_bc, p.e.n_res, p.e.n_ic, p.e.n_bc, pp, j);
-                  db[1 + j] = fmaf(v[u][0][i], x, db[1 + j]);
-                  if (j < nd) db[1 + j] += v[u][1 + j][i];
-                }
-              }
-            }
-          }
+          for (int i = 0; i < UPTS; ++i) db[0] += v[u][0][i];
+          if (p.e.dterms) coord_terms<UPTS>(v[u], xc, u * UPTS, p.e.dterms, p.e.jet_mode, db);
         }
       }
       // done with this A tile: its ordinary shared loads ordered before the next bulk copy
