@@ -32,3 +32,13 @@ def _parity(spec, n_res, n_ic, n_bc, precision, what):
 def test_fp32_gemm_edges(cuda_lib, widths, ff, n_res):
     spec = NetSpec(PDE_NS, 2, 3, widths, ff_m=ff, ff_sigma=1.0, rwf=True)
     _parity(spec, n_res, 0, 33, "fp32", f"fp32 {widths} {n_res}")
+
+
+@pytest.mark.parametrize("precision", ["fp32", "bf16"])
+@pytest.mark.parametrize("pde,widths,n", [
+    (PDE_BURGERS, [40, 16], (61, 2, 1)),          # one feature per thread, sets meeting inside a 4- or 8-point group
+    (PDE_MAXWELL, [104, 16], (20003, 501, 77)),   # several features per thread, a remainder of them
+])
+def test_first_layer_edges(cuda_lib, pde, widths, n, precision):
+    spec = NetSpec(pde, 3 if pde == PDE_MAXWELL else 2, 3 if pde == PDE_MAXWELL else 1, widths, rwf=True)
+    _parity(spec, *n, precision, f"first layer {widths} {n} {precision}")
