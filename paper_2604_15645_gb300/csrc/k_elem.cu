@@ -429,6 +429,51 @@ template <> __device__ __forceinline__ void store4_stream<__nv_bfloat16>(__nv_bf
   __stcs(reinterpret_cast<uint2*>(p), u);
 }
 
+// Temporal causality, first pass: the segment sums of squared residuals.  Each warp keeps
+// its own sums in shared memory, SEG_WORDS floats: lane s owns segment s (at most 32) and
+// adds the warp's 16 points of a tile in order, as compensated FP32 pairs (exact to about
+// 2^-48, like the FP64 sums they become at the end of the block).  The points' squared
+// residuals and segment come from the 16 float4 staged after the sums.  (One thread adding all
+// 64 points of a tile in FP64, with the block waiting at two barriers, was most of the pass:
+// both output passes of a 4x128 network at 17,408 points 0.156 -> 0.062 ms.)
+constexpr int SEG_SUMS = 7 * CAUSAL_MAX;            // 3 equations x (sum, compensation), count
+constexpr int SEG_WORDS = SEG_SUMS + 4 * 16;
+
+__device__ __forceinline__ float4* seg_points(float* sw) { return reinterpret_cast<float4*>(sw + SEG_SUMS); }
+__device__ __forceinline__ void seg_clear(float* sw, int lane) {
+#pragma unroll
+  for (int k = 0; k < 7; ++k) sw[k * CAUSAL_MAX + lane] = 0.f;
+}
+__device__ __forceinline__ void seg_add(float* sw, int lane) {
+  __syncwarp();
+  Acc2 a[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) { a[k].s = sw[(2 * k) * CAUSAL_MAX + lane]; a[k].c = sw[(2 * k + 1) * CAUSAL_MAX + lane]; }
+  float n = sw[6 * CAUSAL_MAX + lane];
+  const float4* pts = seg_points(sw);
+#pragma unroll 4
+  for (int q = 0; q < 16; ++q) {
+    const float4 v = pts[q];
+    const bool mine = __float_as_int(v.w) == lane;
+    a[0].add(mine ? v.x : 0.f); a[1].add(mine ? v.y : 0.f); a[2].add(mine ? v.z : 0.f);
+    n += mine ? 1.f : 0.f;
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) { sw[(2 * k) * CAUSAL_MAX + lane] = a[k].s; sw[(2 * k + 1) * CAUSAL_MAX + lane] = a[k].c; }
+  sw[6 * CAUSAL_MAX + lane] = n;
+  __syncwarp();
+}
+// The block's sums of segment s, column k (3 equations, count): four warps in order.
+__device__ __forceinline__ double seg_total(const float* sw0, int stride, int s, int k) {
+  double t = 0.0;
+  for (int w = 0; w < 4; ++w) {
+    const float* sw = sw0 + w * stride;
+    t += k == 3 ? (double)sw[6 * CAUSAL_MAX + s]
+                : (double)sw[(2 * k) * CAUSAL_MAX + s] + (double)sw[(2 * k + 1) * CAUSAL_MAX + s];
+  }
+  return t;
+}
+
 // One block per 64-point tile (grid-stride).  Warp w takes points 16w..16w+15;
 // lane = 8 * pg + sl: point group pg (4 consecutive points) and feature slice sl
 // (features sl, sl+8, ...).  The 8 slices of a point group combine their partial
@@ -453,13 +498,8 @@ __global__ void __launch_bounds__(OUT_THREADS) k_out_loss(OutArgs a) {
   const int64_t ntiles = a.NP / TILE_PTS;
   Acc2 acc[5];   // compensated FP32 running sums (FP64 is a slow pipe on this part)
   float dbo[3] = {0.f, 0.f, 0.f};                 // output bias gradient (value-row seeds)
-  // temporal causality, first pass: this block's segment sums (3 equations + count),
-  // accumulated by one thread over the tile's points in a fixed order
-  __shared__ double segacc[CAUSAL_MAX][4];
-  __shared__ int s_seg[TILE_PTS];
-  __shared__ float s_rr[TILE_PTS][3];
-  if (a.segpart)
-    for (int i = threadIdx.x; i < CAUSAL_MAX * 4; i += blockDim.x) segacc[i / 4][i % 4] = 0.0;
+  __shared__ __align__(16) float s_seg[OUT_THREADS / 32][SEG_WORDS];   // causality: segment sums per warp
+  if (a.segpart) seg_clear(s_seg[warp], lane);
   for (int64_t T0i = blockIdx.x; T0i < ntiles; T0i += gridDim.x) {
     const int64_t T0 = a.reverse ? ntiles - 1 - T0i : T0i;
     const int64_t cb = T0 * TILE_COLS + q0;        // column of row 0 of the first point
@@ -530,18 +570,9 @@ __global__ void __launch_bounds__(OUT_THREADS) k_out_loss(OutArgs a) {
     if (a.segpart) {   // uniform over the block
       if (sl == 0)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          s_seg[q0 + j] = segj[j];
-          s_rr[q0 + j][0] = rrj[j][0]; s_rr[q0 + j][1] = rrj[j][1]; s_rr[q0 + j][2] = rrj[j][2];
-        }
-      __syncthreads();
-      if (threadIdx.x == 0)
-        for (int q = 0; q < TILE_PTS; ++q)
-          if (s_seg[q] >= 0) {
-            double* sa = segacc[s_seg[q]];
-            sa[0] += s_rr[q][0]; sa[1] += s_rr[q][1]; sa[2] += s_rr[q][2]; sa[3] += 1.0;
-          }
-      __syncthreads();
+        for (int j = 0; j < 4; ++j)
+          seg_points(s_seg[warp])[(q0 & 15) + j] = make_float4(rrj[j][0], rrj[j][1], rrj[j][2], __int_as_float(segj[j]));
+      seg_add(s_seg[warp], lane);
     }
     if (!a.want_grad) continue;
     if (sl == 0) {
@@ -623,7 +654,7 @@ __global__ void __launch_bounds__(OUT_THREADS) k_out_loss(OutArgs a) {
   if (a.segpart) {
     __syncthreads();
     for (int i = threadIdx.x; i < CAUSAL_MAX * 4; i += blockDim.x)
-      a.segpart[(int64_t)blockIdx.x * CAUSAL_MAX * 4 + i] = segacc[i / 4][i % 4];
+      a.segpart[(int64_t)blockIdx.x * CAUSAL_MAX * 4 + i] = seg_total(s_seg[0], SEG_WORDS, i / 4, i % 4);
   }
   if (!a.want_grad) return;
   // block partials of the output layer's dW (warps summed in a fixed order) and bias
@@ -740,9 +771,7 @@ __global__ void __launch_bounds__(OT_THREADS) k_out_loss_tma(const __grid_consta
   uint64_t* full = reinterpret_cast<uint64_t*>(ring + bar_off);
   uint64_t* empty = full + OT_STAGES;
   volatile int* abort_flag = reinterpret_cast<volatile int*>(empty + OT_STAGES);
-  __shared__ double segacc[CAUSAL_MAX][4];
-  __shared__ int s_seg[TILE_PTS];
-  __shared__ float s_rr[TILE_PTS][3];
+  __shared__ __align__(16) float s_seg[OT_CONS / 32][SEG_WORDS];   // causality: segment sums per warp
   __shared__ double sh[OT_CONS / 32];
   __shared__ float shb[OT_CONS / 32];
 
@@ -757,8 +786,7 @@ __global__ void __launch_bounds__(OT_THREADS) k_out_loss_tma(const __grid_consta
   }
   for (int i = threadIdx.x; i < D * w; i += blockDim.x) sW[i] = a.W[i];
   for (int i = threadIdx.x; i < (OT_CONS / 32) * (D + 1) * w; i += blockDim.x) sdw[i] = 0.f;
-  if (a.segpart)
-    for (int i = threadIdx.x; i < CAUSAL_MAX * 4; i += blockDim.x) segacc[i / 4][i % 4] = 0.0;
+  if (a.segpart && warp < OT_CONS / 32) seg_clear(s_seg[warp], lane);
   __syncthreads();
 
   const int64_t ntiles = a.NP / TILE_PTS;
@@ -890,18 +918,9 @@ __global__ void __launch_bounds__(OT_THREADS) k_out_loss_tma(const __grid_consta
     if (a.segpart) {
       if (sl == 0)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          s_seg[q0 + j] = segj[j];
-          s_rr[q0 + j][0] = rrj[j][0]; s_rr[q0 + j][1] = rrj[j][1]; s_rr[q0 + j][2] = rrj[j][2];
-        }
-      cons_sync();
-      if (threadIdx.x == 0)
-        for (int q = 0; q < TILE_PTS; ++q)
-          if (s_seg[q] >= 0) {
-            double* sa = segacc[s_seg[q]];
-            sa[0] += s_rr[q][0]; sa[1] += s_rr[q][1]; sa[2] += s_rr[q][2]; sa[3] += 1.0;
-          }
-      cons_sync();
+        for (int j = 0; j < 4; ++j)
+          seg_points(s_seg[warp])[(q0 & 15) + j] = make_float4(rrj[j][0], rrj[j][1], rrj[j][2], __int_as_float(segj[j]));
+      seg_add(s_seg[warp], lane);
     }
     if (!a.want_grad) continue;
     if (sl == 0) {
@@ -976,7 +995,7 @@ __global__ void __launch_bounds__(OT_THREADS) k_out_loss_tma(const __grid_consta
   if (a.segpart) {
     cons_sync();
     for (int i = threadIdx.x; i < CAUSAL_MAX * 4; i += OT_CONS)
-      a.segpart[(int64_t)blockIdx.x * CAUSAL_MAX * 4 + i] = segacc[i / 4][i % 4];
+      a.segpart[(int64_t)blockIdx.x * CAUSAL_MAX * 4 + i] = seg_total(s_seg[0], SEG_WORDS, i / 4, i % 4);
   }
   if (!a.want_grad) return;
   cons_sync();
@@ -1151,9 +1170,6 @@ __global__ void __launch_bounds__(OT_THREADS, 2) k_out_loss_mma(const __grid_con
   uint64_t* full = reinterpret_cast<uint64_t*>(ring + lay.bar);
   uint64_t* empty = full + OT_STAGES;
   volatile int* abort_flag = reinterpret_cast<volatile int*>(empty + OT_STAGES);
-  __shared__ double segacc[CAUSAL_MAX][4];
-  __shared__ int s_seg[TILE_PTS];
-  __shared__ float s_rr[TILE_PTS][3];
   __shared__ double sh[OT_CONS / 32];
   __shared__ float shb[OT_CONS / 32];
 
@@ -1197,8 +1213,6 @@ __global__ void __launch_bounds__(OT_THREADS, 2) k_out_loss_mma(const __grid_con
     for (int j = 0; j < 4; ++j) sWf[4 * i + j] = q[j];
   }
   for (int i = threadIdx.x; i < 4 * D * (w + 8) + 4 * w; i += blockDim.x) sdw[i] = 0.f;   // sdw and sdb
-  if (a.segpart)
-    for (int i = threadIdx.x; i < CAUSAL_MAX * 4; i += blockDim.x) segacc[i / 4][i % 4] = 0.0;
   __syncthreads();
 
   const int64_t ntiles = a.NP / TILE_PTS;
@@ -1254,6 +1268,10 @@ __global__ void __launch_bounds__(OT_THREADS, 2) k_out_loss_mma(const __grid_con
   float* sU = reinterpret_cast<float*>(scr);                                  // [16 points][D][4]
   __nv_bfloat16* sUd = reinterpret_cast<__nv_bfloat16*>(scr + 768);          // [hi/lo][4 rows][D][16 points]
   uint8_t* sUb = scr + 1536;                                                   // [4 rows][16 points][16 k] bf16
+  // causality: segment sums of this warp, in the seed scratch (the first causal pass takes no gradient)
+  static_assert(OM_SCRATCH - 768 >= SEG_WORDS * (int)sizeof(float), "segment sums fit in the seed scratch");
+  float* sseg = reinterpret_cast<float*>(scr + 768);
+  if (a.segpart) seg_clear(sseg, lane);
   const uint32_t stg = smem_u32(ring + lay.stg);                              // Zbar_L chunk staging
   const uint32_t sWA_u = smem_u32(sWA);
   const uint32_t sUd_u = smem_u32(sUd);
@@ -1504,18 +1522,8 @@ __global__ void __launch_bounds__(OT_THREADS, 2) k_out_loss_mma(const __grid_con
       }
     }
     if (a.segpart) {   // uniform over the block
-      if (lane < 16) {
-        s_seg[p0 + lane] = seg;
-        s_rr[p0 + lane][0] = rr[0]; s_rr[p0 + lane][1] = rr[1]; s_rr[p0 + lane][2] = rr[2];
-      }
-      cons_sync();
-      if (threadIdx.x == 0)
-        for (int q = 0; q < TILE_PTS; ++q)
-          if (s_seg[q] >= 0) {
-            double* sa = segacc[s_seg[q]];
-            sa[0] += s_rr[q][0]; sa[1] += s_rr[q][1]; sa[2] += s_rr[q][2]; sa[3] += 1.0;
-          }
-      cons_sync();
+      if (lane < 16) seg_points(sseg)[lane] = make_float4(rr[0], rr[1], rr[2], __int_as_float(seg));
+      seg_add(sseg, lane);
     }
     if (a.want_grad) {
     __syncwarp();
@@ -1549,7 +1557,8 @@ __global__ void __launch_bounds__(OT_THREADS, 2) k_out_loss_mma(const __grid_con
   if (a.segpart) {
     cons_sync();
     for (int i = threadIdx.x; i < CAUSAL_MAX * 4; i += OT_CONS)
-      a.segpart[(int64_t)blockIdx.x * CAUSAL_MAX * 4 + i] = segacc[i / 4][i % 4];
+      a.segpart[(int64_t)blockIdx.x * CAUSAL_MAX * 4 + i] =
+          seg_total(reinterpret_cast<const float*>(ring + lay.stg + 768), OM_SCRATCH / 4, i / 4, i % 4);
   }
   if (!a.want_grad) return;
   cons_sync();
@@ -1927,42 +1936,69 @@ void launch_finalize_loss(const double* part, int nblocks, int64_t n_res, int64_
 }
 
 // ------------------------------------------------------------------------------------
-// Temporal causality (Sec. 2.6.8, Eqs. 20-21).  Thread (i, e) sums segment i's
-// equation-e partials over the blocks in order; thread 0 then forms the segment
-// losses L^i = sum_e S_ie / N_i, omega_1 = 1, omega_i = exp(-eps sum_{k<i} L^k), the
-// weighted PDE term (1/M) sum_i omega_i L^i (and per equation), and the seed scales.
+// Temporal causality (Sec. 2.6.8, Eqs. 20-21).  The blocks' partials are summed by FC_G
+// threads per (segment, column), combined in order; then the segment losses
+// L^i = sum_e S_ie / N_i, omega_1 = 1, omega_i = exp(-eps sum_{k<i} L^k) (one thread per
+// segment once the running sums stand), the weighted PDE term (1/M) sum_i omega_i L^i
+// (and per equation), and the seed scales.  One block, bound by latency: the sums run
+// FC_G wide and the exponentials side by side instead of one after the other.
 // ------------------------------------------------------------------------------------
-__global__ void k_finalize_causal(const double* segpart, const double* losspart, int nblocks, int M, double eps,
-                                  int64_t n_ic, int64_t n_bc, double lam_pde, double lam_ic, double lam_bc,
-                                  double lam_seed, double* out, double* omega, float* scale, int* status) {
+constexpr int FC_G = 4, FC_COLS = CAUSAL_MAX * 4 + 2;   // segment columns, then the IC and BC sums
+
+__global__ void __launch_bounds__(FC_G * FC_COLS)
+    k_finalize_causal(const double* __restrict__ segpart, const double* __restrict__ losspart, int nblocks, int M,
+                      double eps, int64_t n_ic, int64_t n_bc, double lam_pde, double lam_ic, double lam_bc,
+                      double lam_seed, double* out, double* omega, float* scale, int* status) {
+  __shared__ double part[FC_G][FC_COLS];
   __shared__ double S[CAUSAL_MAX][4];
-  __shared__ double ib[2];
+  __shared__ double ib[2], L[CAUSAL_MAX], cum[CAUSAL_MAX];
   const int t = threadIdx.x;
-  if (t < M * 4) {
+  {
+    const int c = t % FC_COLS, g = t / FC_COLS;
+    const bool seg = c < CAUSAL_MAX * 4;
+    const double* src = seg ? segpart + c : losspart + 3 + (c - CAUSAL_MAX * 4);
+    const int stride = seg ? CAUSAL_MAX * 4 : 8;
     double s = 0.0;
-    for (int b = 0; b < nblocks; ++b) s += segpart[(int64_t)b * CAUSAL_MAX * 4 + t];
-    S[t / 4][t % 4] = s;
-  } else if (t >= 128 && t < 130) {
-    double s = 0.0;
-    for (int b = 0; b < nblocks; ++b) s += losspart[(int64_t)b * 8 + 3 + (t - 128)];
-    ib[t - 128] = s;
+    if (!seg || c < M * 4)
+#pragma unroll 8
+      for (int b = g; b < nblocks; b += FC_G) s += src[(int64_t)b * stride];
+    part[g][c] = s;
+  }
+  __syncthreads();
+  if (t < FC_COLS) {
+    double s = part[0][t];
+    for (int g = 1; g < FC_G; ++g) s += part[g][t];
+    if (t < CAUSAL_MAX * 4) S[t / 4][t % 4] = s;
+    else ib[t - CAUSAL_MAX * 4] = s;
+  }
+  __syncthreads();
+  if (t < M) {
+    const double n = S[t][3];
+    double Li = 0.0;
+    for (int e = 0; e < 3; ++e) {
+      const double le = n > 0.0 ? S[t][e] / n : 0.0;
+      S[t][e] = le;
+      Li += le;
+    }
+    L[t] = Li;
+  }
+  __syncthreads();
+  if (t == 0) {
+    double c = 0.0;
+    for (int i = 0; i < M; ++i) { cum[i] = c; c += L[i]; }
+  }
+  __syncthreads();
+  if (t < M) {
+    const double n = S[t][3], wi = exp(-eps * cum[t]);   // omega_i from the segments before i
+    omega[t] = wi;
+    scale[t] = n > 0.0 ? (float)(lam_seed * wi / (M * n)) : 0.f;
+    for (int e = 0; e < 3; ++e) S[t][e] = wi * S[t][e] / M;
   }
   __syncthreads();
   if (t != 0) return;
-  double cum = 0.0, pe[3] = {0.0, 0.0, 0.0};
-  for (int i = 0; i < M; ++i) {
-    const double n = S[i][3];
-    const double w = exp(-eps * cum);             // omega_i from the segments before i
-    double Li = 0.0;
-    for (int e = 0; e < 3; ++e) {
-      const double le = n > 0.0 ? S[i][e] / n : 0.0;
-      pe[e] += w * le / M;
-      Li += le;
-    }
-    cum += Li;
-    omega[i] = w;
-    scale[i] = n > 0.0 ? (float)(lam_seed * w / (M * n)) : 0.f;
-  }
+  double pe[3] = {0.0, 0.0, 0.0};
+  for (int i = 0; i < M; ++i)
+    for (int e = 0; e < 3; ++e) pe[e] += S[i][e];
   const double lic = n_ic ? ib[0] / n_ic : 0.0, lbc = n_bc ? ib[1] / n_bc : 0.0;
   const double lpde = pe[0] + pe[1] + pe[2];
   const double tot = lam_pde * lpde + lam_ic * lic + lam_bc * lbc;
@@ -1973,7 +2009,7 @@ __global__ void k_finalize_causal(const double* segpart, const double* losspart,
 void launch_finalize_causal(const double* segpart, const double* losspart, int nblocks, int M, double eps,
                             int64_t n_ic, int64_t n_bc, double lam_pde, double lam_ic, double lam_bc, double lam_seed,
                             double* out, double* omega, float* scale, int* status, cudaStream_t st) {
-  k_finalize_causal<<<1, 256, 0, st>>>(segpart, losspart, nblocks, M, eps, n_ic, n_bc, lam_pde, lam_ic, lam_bc,
+  k_finalize_causal<<<1, FC_G * FC_COLS, 0, st>>>(segpart, losspart, nblocks, M, eps, n_ic, n_bc, lam_pde, lam_ic, lam_bc,
                                        lam_seed, out, omega, scale, status);
 }
 

@@ -42,3 +42,27 @@ def test_fp32_gemm_edges(cuda_lib, widths, ff, n_res):
 def test_first_layer_edges(cuda_lib, pde, widths, n, precision):
     spec = NetSpec(pde, 3 if pde == PDE_MAXWELL else 2, 3 if pde == PDE_MAXWELL else 1, widths, rwf=True)
     _parity(spec, *n, precision, f"first layer {widths} {n} {precision}")
+
+
+@pytest.mark.parametrize("precision,width", [("fp32", 13), ("bf16", 64), ("bf16", 320)])
+@pytest.mark.parametrize("segments,n_res", [(32, 1000), (5, 3)])
+def test_causal_segment_sums(cuda_lib, precision, width, segments, n_res):
+    """All 32 segments, and segments without points, in each of the three output kernels."""
+    import oracle
+    from paper_2604_15645_gb300 import api
+    spec = NetSpec(PDE_BURGERS, 2, 1, [width, width])
+    p = init_params(spec, 81, 0.2)
+    b = make_batch(PDE_BURGERS, n_res, 40, 30, 82, 83)
+    net = api.PinnNet.from_spec(spec, precision)
+    net.set_causal(segments, 1.5)
+    t, g = net.loss_grad(torch.tensor(p, device="cuda"), api.DeviceBatch.from_host(b), api.make_problem(0.05, 1.0, 0.5, 2.0))
+    torch.cuda.synchronize()
+    assert net.status_poll() == 0
+    cz = dict(segments=segments, eps=1.5, t_index=1, t0=0.0, t1=1.0)
+    terms, rg = oracle.loss_and_grad(oracle.Model.from_spec(spec), p, None, b, 0.05, (1.0, 0.5, 2.0), causal=cz)
+    tol = TOL[precision]
+    t = t.cpu().numpy()
+    assert abs(t[0] - terms["total"]) <= tol * abs(terms["total"])
+    assert abs(t[1] - terms["pde"]) <= tol * abs(terms["pde"])
+    assert np.linalg.norm(g.cpu().numpy() - rg) <= tol * np.linalg.norm(rg)
+    assert np.allclose(net.causal_weights().cpu().numpy(), terms["causal_weights"], rtol=10 * tol)
