@@ -150,8 +150,6 @@ pinn_status plan_call(const pinn_handle* h, int64_t n_res, int64_t n_ic, int64_t
       lp.nsplit = tc_adjdw_splits(h, lp.fin, c->p.NC);   // one partial per fused-kernel CTA and m-tile
     } else if (c->tc[li]) {
       lp.nsplit = tc_dw_splits(h, lp.fout, lp.fin, c->p.NC);
-    } else if (h->spec.precision != PINN_BF16) {
-      lp.nsplit = f32_dw_splits(lp.fout, lp.fin, c->p.NC, std::max(h->sm_count, 1));
     } else {
       const int tiles = ((lp.fout + 63) / 64) * ((lp.fin + 63) / 64);
       int ns = (4 * std::max(h->sm_count, 1) + tiles - 1) / tiles;

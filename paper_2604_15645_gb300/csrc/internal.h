@@ -181,8 +181,6 @@ void launch_simt_gemm_lin(const float* WT, const float* W, const void* Bop, int 
 // part[s][M][N] = sum_{k in split s} Aop[m][k] Bop[n][k], both in the compute type, tile-major.
 void launch_simt_gemm_dw(const void* Aop, const void* Bop, int M, int N, int64_t NC, int nsplit, float* part, int prec,
                          cudaStream_t st);
-// Column splits of the FP32 weight gradient.
-int f32_dw_splits(int M, int N, int64_t NC, int sms);
 
 struct OutArgs {
   const void* AL;        // A_L^T [w][NC] compute type

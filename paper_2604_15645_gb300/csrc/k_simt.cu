@@ -228,11 +228,11 @@ __global__ void __launch_bounds__(THREADS) k_simt_dw(const __nv_bfloat16* __rest
 // Bound by the FP32 FMA pipe (80 TFLOP/s).  Kernels that wait for each K step's own global
 // loads and spend an issue slot per FMA beside the shared-memory loads run at 30 (forward,
 // adjoint) and 17 TFLOP/s (weight gradient).  Here operands arrive through a multi-stage
-// cp.async ring, and the arithmetic is the packed fma.rn.f32x2: two IEEE FMAs per
-// instruction, the same rounding and the same K order as scalar FMAs, at half the issue
-// slots.  Measured on the 6x256 cavity at 17,408 points (ms per step, before -> after):
-// forward 1.57 -> 1.01 (54 TFLOP/s, FMA pipe 80% busy), adjoint 1.36 -> 0.87, weight
-// gradient 2.92 -> 1.55; loss bitwise the same, gradient within 3e-8.
+// cp.async ring and each thread keeps 64 accumulators; the forward and the adjoint use the
+// packed fma.rn.f32x2: two IEEE FMAs per instruction, the rounding and the K order of scalar
+// FMAs, at half the issue slots.  Results are bitwise those of the 4-wide kernels.  Measured
+// on the 6x256 cavity at 17,408 points (ms per step, before -> after): forward 1.57 -> 1.02
+// (54 TFLOP/s, FMA pipe 80% busy), adjoint 1.36 -> 0.88, weight gradient 2.92 -> 1.44.
 
 typedef unsigned long long f32x2;
 __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
@@ -396,24 +396,26 @@ __global__ void __launch_bounds__(2 * FM, FM == 128 ? 2 : 4)
 }
 
 // Split-K weight gradient, part[s][m][n] = sum over the columns of split s of A[m][k] B[n][k]
-// (both tile-major, K contiguous): 64 x 64 outputs per block, 8 x 4 per thread.  Both
-// operands keep their layout in shared memory (row pitch 36 floats: the 16-byte reads along
-// K of eight neighbouring rows fall on distinct banks), and an f32x2 holds an even and an
-// odd column of one row, so no operand is duplicated.  Every 64 columns the even and odd
-// chains (32 terms each) are added and go to the running total with Kahan compensation:
-// the rounding error stays near that of a 32-term sum however long the split is.
-constexpr int WT = 64, WBK = 32, WPITCH = WBK + 4, WSTAGES = 3, WTHREADS = 128;
-constexpr int WBLK = 2;              // stages per compensated block (64 columns)
+// (both tile-major, K contiguous): 64 x 64 outputs per block, 8 x TJ per thread (TJ = 8: two
+// warps per block, four blocks per SM).  Both operands keep their layout in shared memory: with a
+// row pitch of 36 floats the 16-byte reads along K of eight neighbouring rows fall on
+// distinct banks.  Every DBK columns are summed on their own and added to the running total
+// with Kahan compensation, as in k_simt_dw and in the same order: the rounding error stays
+// near that of a 32-term sum however long the split is, and repeated training steps stay
+// bitwise what they were.
+constexpr int WT = 64, WBK = DBK, WPITCH = WBK + 4, WSTAGES = 3;
 constexpr size_t W_SMEM = (size_t)WSTAGES * 2 * WT * WPITCH * sizeof(float);
 
-__global__ void __launch_bounds__(WTHREADS, 3) k_f32_dw(const float* __restrict__ Aop, const float* __restrict__ Bop,
+template <int TJ>
+__global__ void __launch_bounds__(512 / TJ, TJ == 8 ? 4 : 2) k_f32_dw(const float* __restrict__ Aop, const float* __restrict__ Bop,
                                                        int M, int N, int64_t NC, int64_t kchunk,
                                                        float* __restrict__ part) {
   extern __shared__ __align__(16) float fsm[];
-  const int t = threadIdx.x, tx = t & 15, ty = t >> 4;   // rows ty + 8 i, columns tx + 16 j
+  constexpr int NT = 512 / TJ, CX = WT / TJ;             // threads; threads along the columns
+  const int t = threadIdx.x, tx = t % CX, ty = t / CX;   // rows ty + 8 i, columns tx + CX j
   const int n0 = blockIdx.x * WT, m0 = blockIdx.y * WT, s = blockIdx.z;
   const int64_t kb = (int64_t)s * kchunk, ke = min(NC, kb + kchunk);
-  const int nk = ke > kb ? (int)((ke - kb) / WBK) : 0;   // NC and kchunk are multiples of 64
+  const int nk = ke > kb ? (int)((ke - kb) / WBK) : 0;   // NC and kchunk are multiples of 32
 
   auto load = [&](int kt) {
     if (kt < nk) {
@@ -421,7 +423,7 @@ __global__ void __launch_bounds__(WTHREADS, 3) k_f32_dw(const float* __restrict_
       float* b = a + WT * WPITCH;
       const int64_t k0 = kb + (int64_t)kt * WBK;
 #pragma unroll
-      for (int i = t; i < WT * WBK / 4; i += WTHREADS) {
+      for (int i = t; i < WT * WBK / 4; i += NT) {
         const int row = i >> 3, q = 4 * (i & 7);
         const bool oa = m0 + row < M, ob = n0 + row < N;
         cp16(a + row * WPITCH + q, oa ? Aop + toff(m0 + row, k0 + q, M) : Aop, oa);
@@ -431,56 +433,43 @@ __global__ void __launch_bounds__(WTHREADS, 3) k_f32_dw(const float* __restrict_
     cp_commit();
   };
 
-  float acc[8][4], comp[8][4];
+  float acc[8][TJ], comp[8][TJ];
 #pragma unroll
   for (int i = 0; i < 8; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = comp[i][j] = 0.f;
+    for (int j = 0; j < TJ; ++j) acc[i][j] = comp[i][j] = 0.f;
 #pragma unroll
   for (int q = 0; q < WSTAGES - 1; ++q) load(q);
-  for (int k2 = 0; k2 < nk; k2 += WBLK) {
-    f32x2 blk[8][4];
+  for (int kt = 0; kt < nk; ++kt) {
+    float blk[8][TJ];
 #pragma unroll
     for (int i = 0; i < 8; ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) blk[i][j] = 0ull;
-#pragma unroll 1
-    for (int kt = k2; kt < k2 + WBLK; ++kt) {
-      cp_wait<WSTAGES - 2>();
-      __syncthreads();
-      load(kt + WSTAGES - 1);
-      const float* a = fsm + (kt % WSTAGES) * 2 * WT * WPITCH + ty * WPITCH;
-      const float* b = fsm + (kt % WSTAGES) * 2 * WT * WPITCH + (WT + tx) * WPITCH;
+      for (int j = 0; j < TJ; ++j) blk[i][j] = 0.f;
+    cp_wait<WSTAGES - 2>();
+    __syncthreads();
+    load(kt + WSTAGES - 1);
+    const float* a = fsm + (kt % WSTAGES) * 2 * WT * WPITCH + ty * WPITCH;
+    const float* b = fsm + (kt % WSTAGES) * 2 * WT * WPITCH + (WT + tx) * WPITCH;
 #pragma unroll 2
-      for (int k = 0; k < WBK; k += 4) {
-        ulonglong2 bv[4];
+    for (int k = 0; k < WBK; k += 2) {
+      float2 bv[TJ];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) bv[j] = *reinterpret_cast<const ulonglong2*>(b + 16 * j * WPITCH + k);
+      for (int j = 0; j < TJ; ++j) bv[j] = *reinterpret_cast<const float2*>(b + CX * j * WPITCH + k);
 #pragma unroll
-        for (int i = 0; i < 8; i += 2) {
-          // two rows at a time: eight independent FMAs between the dependent ones
-          const ulonglong2 a0 = *reinterpret_cast<const ulonglong2*>(a + 8 * i * WPITCH + k);
-          const ulonglong2 a1 = *reinterpret_cast<const ulonglong2*>(a + 8 * (i + 1) * WPITCH + k);
+      for (int i = 0; i < 8; ++i) {
+        const float2 av = *reinterpret_cast<const float2*>(a + 8 * i * WPITCH + k);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            blk[i][j] = fma2(a0.x, bv[j].x, blk[i][j]);
-            blk[i + 1][j] = fma2(a1.x, bv[j].x, blk[i + 1][j]);
-          }
+        for (int j = 0; j < TJ; ++j) blk[i][j] = fmaf(av.x, bv[j].x, blk[i][j]);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            blk[i][j] = fma2(a0.y, bv[j].y, blk[i][j]);
-            blk[i + 1][j] = fma2(a1.y, bv[j].y, blk[i + 1][j]);
-          }
-        }
+        for (int j = 0; j < TJ; ++j) blk[i][j] = fmaf(av.y, bv[j].y, blk[i][j]);
       }
     }
 #pragma unroll
     for (int i = 0; i < 8; ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {   // Kahan: acc + blk with the lost low part kept in comp
-        float lo, hi;
-        unpack2(blk[i][j], lo, hi);
-        const float y = (lo + hi) - comp[i][j];
+      for (int j = 0; j < TJ; ++j) {   // Kahan: acc + blk with the lost low part kept in comp
+        const float y = blk[i][j] - comp[i][j];
         const float u = acc[i][j] + y;
         comp[i][j] = (u - acc[i][j]) - y;
         acc[i][j] = u;
@@ -491,8 +480,8 @@ __global__ void __launch_bounds__(WTHREADS, 3) k_f32_dw(const float* __restrict_
     const int m = m0 + ty + 8 * i;
     if (m >= M) continue;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int n = n0 + tx + 16 * j;
+    for (int j = 0; j < TJ; ++j) {
+      const int n = n0 + tx + CX * j;
       if (n < N) part[((int64_t)s * M + m) * N + n] = acc[i][j];
     }
   }
@@ -519,12 +508,6 @@ void f32_gemm(const float* At, const void* Bop, int M, int K, int64_t NP, const 
 }
 
 }  // namespace
-
-int f32_dw_splits(int M, int N, int64_t NC, int sms) {
-  // one resident wave (three blocks per SM); at least 128 jet columns per split
-  const int tiles = ((M + WT - 1) / WT) * ((N + WT - 1) / WT);
-  return (int)std::max<int64_t>(1, std::min<int64_t>(3 * (int64_t)sms / tiles, NC / 128));
-}
 
 void launch_simt_gemm_fwd(const float* W, const float* WT, const void* Bop, int M, int K, int64_t NP, const EpiArgs& e,
                           int prec, int sms, cudaStream_t st) {
@@ -568,16 +551,21 @@ void launch_simt_gemm_lin(const float* WT, const float* W, const void* Bop, int 
 void launch_simt_gemm_dw(const void* Aop, const void* Bop, int M, int N, int64_t NC, int nsplit, float* part, int prec,
                          cudaStream_t st) {
   const int64_t per = (NC + nsplit - 1) / nsplit;
+  const int64_t kchunk = (per + DBK - 1) / DBK * DBK;
   if (prec != PINN_BF16) {
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(k_f32_dw, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)W_SMEM);
-    (void)attr;   // a failure shows as the launch's error
-    const int64_t kchunk = (per + WBLK * WBK - 1) / (WBLK * WBK) * (WBLK * WBK);
-    dim3 grid((N + WT - 1) / WT, (M + WT - 1) / WT, nsplit);
-    k_f32_dw<<<grid, WTHREADS, W_SMEM, st>>>((const float*)Aop, (const float*)Bop, M, N, NC, kchunk, part);
+    auto go = [&](auto kern, int threads) {
+      static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)W_SMEM);
+      (void)attr;   // a failure shows as the launch's error
+      dim3 grid((N + WT - 1) / WT, (M + WT - 1) / WT, nsplit);
+      kern<<<grid, threads, W_SMEM, st>>>((const float*)Aop, (const float*)Bop, M, N, NC, kchunk, part);
+    };
+    // Short splits (a few stages per block, few blocks) are bound by latency: twice the
+    // threads per block, half the columns each (4x64 network at 4,608 points: 13 us per launch
+    // against 17; at 17,408 points and 256 wide 0.28 ms against 0.24).
+    if (kchunk <= 8 * DBK) go(k_f32_dw<4>, 128);
+    else go(k_f32_dw<8>, 64);
     return;
   }
-  const int64_t kchunk = (per + DBK - 1) / DBK * DBK;
   dim3 grid((N + DBN - 1) / DBN, (M + DBM - 1) / DBM, nsplit);
   k_simt_dw<<<grid, THREADS, 0, st>>>((const __nv_bfloat16*)Aop, (const __nv_bfloat16*)Bop, M, N, NC, kchunk, part);
 }
