@@ -487,6 +487,16 @@ __global__ void __launch_bounds__(512 / TJ, TJ == 8 ? 4 : 2) k_f32_dw(const floa
   }
 }
 
+template <int TJ>
+void f32_dw_launch(const void* Aop, const void* Bop, int M, int N, int64_t NC, int nsplit, int64_t kchunk, float* part,
+                   cudaStream_t st) {
+  static const cudaError_t attr =
+      cudaFuncSetAttribute(k_f32_dw<TJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)W_SMEM);
+  (void)attr;   // a failure shows as the launch's error
+  dim3 grid((N + WT - 1) / WT, (M + WT - 1) / WT, nsplit);
+  k_f32_dw<TJ><<<grid, 512 / TJ, W_SMEM, st>>>((const float*)Aop, (const float*)Bop, M, N, NC, kchunk, part);
+}
+
 template <int FM, int EPI, bool SINE>
 void f32_gemm_launch(const float* At, const void* Bop, int M, int K, int64_t NP, const EpiArgs& e, cudaStream_t st) {
   auto kern = k_f32_gemm<FM, EPI, SINE>;
@@ -553,17 +563,11 @@ void launch_simt_gemm_dw(const void* Aop, const void* Bop, int M, int N, int64_t
   const int64_t per = (NC + nsplit - 1) / nsplit;
   const int64_t kchunk = (per + DBK - 1) / DBK * DBK;
   if (prec != PINN_BF16) {
-    auto go = [&](auto kern, int threads) {
-      static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)W_SMEM);
-      (void)attr;   // a failure shows as the launch's error
-      dim3 grid((N + WT - 1) / WT, (M + WT - 1) / WT, nsplit);
-      kern<<<grid, threads, W_SMEM, st>>>((const float*)Aop, (const float*)Bop, M, N, NC, kchunk, part);
-    };
     // Short splits (a few stages per block, few blocks) are bound by latency: twice the
     // threads per block, half the columns each (4x64 network at 4,608 points: 13 us per launch
     // against 17; at 17,408 points and 256 wide 0.28 ms against 0.24).
-    if (kchunk <= 8 * DBK) go(k_f32_dw<4>, 128);
-    else go(k_f32_dw<8>, 64);
+    if (kchunk <= 8 * DBK) f32_dw_launch<4>(Aop, Bop, M, N, NC, nsplit, kchunk, part, st);
+    else f32_dw_launch<8>(Aop, Bop, M, N, NC, nsplit, kchunk, part, st);
     return;
   }
   dim3 grid((N + DBN - 1) / DBN, (M + DBM - 1) / DBM, nsplit);

@@ -28,6 +28,7 @@ def _parity(spec, n_res, n_ic, n_bc, precision, what):
     ([66, 130, 17], 5, 95),        # widths past a 64- and a 128-feature block, M not a multiple of 4
     ([64, 128, 64], 8, 4096),      # full blocks, 64-feature blocks at this size
     ([80, 72], 24, 9800),          # the smallest sizes that take 128-feature blocks
+    ([64], 32, 30000),             # long weight-gradient splits (the narrow form of the kernel's sums)
 ])
 def test_fp32_gemm_edges(cuda_lib, widths, ff, n_res):
     spec = NetSpec(PDE_NS, 2, 3, widths, ff_m=ff, ff_sigma=1.0, rwf=True)
