@@ -112,6 +112,7 @@ struct CallPlan {
   bool fused_db[PINN_MAX_HIDDEN + 1];  // layer li's bias partials come from a fused adjoint epilogue
   bool out_db = false;                 // the last hidden layer's bias partials come from the output/loss kernel
   int nbpart[PINN_MAX_HIDDEN + 1];     // bias partial count of layer li
+  bool fwd_all = false;                // one kernel runs every hidden GEMM layer's forward
   bool pm = false;                     // TF32 on tensor cores: point-major operand copies
   size_t apm[2] = {0, 0};              // point-major A_l, buffer l % 2 ([NC][fin] FP32)
   size_t zbpm[2] = {0, 0};             // point-major adjoints, ping-pong like Zbar
@@ -133,6 +134,7 @@ pinn_status plan_call(const pinn_handle* h, int64_t n_res, int64_t n_ic, int64_t
     for (int li = 0; li < L1; ++li) c->tc[li] = c->tc[li] && all;
     c->pm = all && h->first_gemm < h->L;
   }
+  c->fwd_all = tc_fwd_all_supported(h, c->p.NC);
   for (int li = 0; li < L1; ++li) c->fused[li] = c->tc[li] && tc_adjdw_supported(h, li, c->p.NC);
   for (int li = 0; li < L1; ++li) {
     LayerPlan lp = h->layers[li];
@@ -280,6 +282,16 @@ struct Pass {
     const Plan& p = cp.p;
     const int L = h->L, prec = h->spec.precision;
     const bool sine = h->act == PINN_ACT_SINE;
+    if (cp.fwd_all && !h->tc_batch) {   // (a grouped step collects the layers' own launches)
+      if (li > h->first_gemm) return PINN_OK;
+      TcFwdLayer y[PINN_MAX_HIDDEN];
+      for (int k = li; k < L; ++k)
+        y[k - li] = TcFwdLayer{ws + cp.lay[k].wc, ws + cp.lay[k].wlo, bias(k), ws + p.A[k + 1], cp.lay[k].fin, cp.lay[k].fout};
+      PhaseScope ps(h, st, PH_FWD, 1);
+      // the tile order of the per-layer path's last layer, which the output stage runs against
+      return tc_gemm_fwd_all(h, y, L - li, ws + p.A[li], ws + p.Alo[li], ws + p.Alo[L], p.NC, h->jet_mode,
+                             ((L - 1 - li) % 2 == 0) ? 1 : 0, want_grad ? 1 : 0, st);
+    }
     EpiArgs e{};
     e.bias = bias(li); e.out = ws + p.A[li + 1];
     e.alo_out = p.lo ? ws + p.Alo[li + 1] : nullptr;

@@ -23,6 +23,7 @@
 #include <cstring>
 
 #include "internal.h"
+#include "ptx.cuh"
 
 namespace pinn {
 
@@ -63,6 +64,52 @@ __device__ __forceinline__ void jet_fwd(const float z[4], float a[4], int mode) 
     const float tpp = -2.f * t * tp;
     const float q = z[1] * z[1] + (mode == JET_NS ? z[2] * z[2] : 0.f);
     a[3] = fmaf(tpp, q, tp * z[3]);
+  }
+}
+
+// jet_fwd<true> of two points at once in packed FP32 (bitwise the same per point): the
+// scalar rule spends about 75 issue slots per point and was most of the forward epilogue
+// (4,800 cycles per 128 x 64-point job, two warps per scheduler); this one takes about 17.
+// The exponent is scaled once by -2 log2(e) (the factor -2 is exact), and the powers of two
+// of t' = 4 e r^2 and t'' = -2 t t' are folded into exact doublings.
+__device__ __forceinline__ float ex2_approx(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float rcp_approx(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ void tanh_fast2(f32x2 z, f32x2& t, f32x2& tp) {
+  constexpr float C = -2.f * 1.4426950408889634f;   // -2 log2(e)
+  float z0, z1;
+  unpack2(z, z0, z1);
+  const f32x2 e = pack2(ex2_approx(fabsf(z0) * C), ex2_approx(fabsf(z1) * C));
+  const f32x2 one = dup2(1.f);
+  float d0, d1;
+  unpack2(add2(one, e), d0, d1);
+  const f32x2 r = pack2(rcp_approx(d0), rcp_approx(d1));
+  float t0, t1;
+  unpack2(mul2(fma2(e, dup2(-1.f), one), r), t0, t1);   // (1 - e) r, >= 0
+  t = pack2(__uint_as_float(__float_as_uint(t0) | (__float_as_uint(z0) & 0x80000000u)),
+            __uint_as_float(__float_as_uint(t1) | (__float_as_uint(z1) & 0x80000000u)));
+  const f32x2 r2 = add2(r, r);
+  tp = mul2(mul2(e, r2), r2);
+}
+template <int MODE>
+__device__ __forceinline__ void jet_fwd2(const f32x2 z[4], f32x2 a[4]) {
+  f32x2 t, tp;
+  tanh_fast2(z[0], t, tp);
+  a[0] = t;
+  a[1] = mul2(tp, z[1]);
+  a[2] = mul2(tp, z[2]);
+  a[3] = mul2(tp, z[3]);
+  if (MODE != JET_MAXWELL) {
+    const f32x2 tpp = mul2(mul2(t, dup2(-2.f)), tp);
+    const f32x2 q = (MODE == JET_NS) ? fma2(z[1], z[1], mul2(z[2], z[2])) : mul2(z[1], z[1]);
+    a[3] = fma2(tpp, q, a[3]);
   }
 }
 

@@ -234,20 +234,6 @@ __global__ void __launch_bounds__(THREADS) k_simt_dw(const __nv_bfloat16* __rest
 // on the 6x256 cavity at 17,408 points (ms per step, before -> after): forward 1.57 -> 1.02
 // (54 TFLOP/s, FMA pipe 80% busy), adjoint 1.36 -> 0.88, weight gradient 2.92 -> 1.44.
 
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
-  f32x2 d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ f32x2 dup2(float x) {
-  f32x2 d;
-  asm("mov.b64 %0, {%1, %1};" : "=l"(d) : "f"(x));
-  return d;
-}
-__device__ __forceinline__ void unpack2(f32x2 v, float& x, float& y) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
-}
 // 16- / 4-byte asynchronous copies global -> shared; `ok` false writes zeros (nothing is read).
 __device__ __forceinline__ void cp16(float* dst, const float* src, bool ok) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(ok ? 16 : 0)

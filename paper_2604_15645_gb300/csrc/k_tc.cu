@@ -35,6 +35,7 @@
 #include <algorithm>
 #include <cstdio>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include "jet.cuh"
@@ -157,6 +158,31 @@ __device__ __forceinline__ void store_pm8(float* pm, int64_t c0, int M, int m, c
   for (int r = 0; r < 4; ++r)
 #pragma unroll
     for (int i = 0; i < 8; ++i) pm[(c0 + 64 * r + i) * M + m] = v[r][i];
+}
+
+// Forward epilogue of 16 points (accumulators v[row][point]) in packed pairs: bias, tanh
+// jet, BF16 rounding (hi, two points per word) and the value row's low half (lo).
+template <int MODE>
+__device__ __forceinline__ void fwd_pairs(const float (&v)[4][16], float bias, uint32_t (&hi)[4][8], uint32_t (&lo)[8],
+                                          uint32_t keep) {
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    f32x2 z[4], a[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) z[r] = pack2(v[r][2 * i], v[r][2 * i + 1]);
+    z[0] = add2(z[0], dup2(bias));
+    jet_fwd2<MODE>(z, a);
+    float x0, x1;
+#pragma unroll
+    for (int r = 3; r >= 0; --r) {
+      unpack2(a[r], x0, x1);
+      const __nv_bfloat162 q = __floats2bfloat162_rn(x0, x1);
+      hi[r][i] = *reinterpret_cast<const uint32_t*>(&q) & keep;
+    }
+    const __nv_bfloat162 q = __floats2bfloat162_rn(x0 - __uint_as_float(hi[0][i] << 16),
+                                                   x1 - __uint_as_float(hi[0][i] & 0xffff0000u));
+    lo[i] = *reinterpret_cast<const uint32_t*>(&q) & keep;
+  }
 }
 
 // Coordinate terms of a raw first layer's weight gradient, dW_ij = sum_points zbar x_j +
@@ -1344,6 +1370,437 @@ pinn_status launch_adjdw_group(pinn_handle* h, const TcGroupEntry* d_tab, int n,
 }
 
 }  // namespace
+
+// ==== the whole hidden forward in one kernel (BF16 tanh, every width <= 256) ===========
+//
+// Layer by layer, a 256-wide forward launch is bound by the data it moves between L2 and
+// the SMs: the weights are re-streamed for every column tile, and the jets (with their
+// value-row low halves) go out and come back once per layer.  Here a CTA takes one column
+// tile (64 points) through every hidden GEMM layer: the tile's jets stay in shared memory,
+// in the MN-major swizzled boxes that the MMAs read as their B operand, and each
+// layer's epilogue writes its outputs back into them.  What leaves the SM is A_l (for the
+// reverse sweep; bulk tensor stores straight from those boxes; nothing in a loss-only
+// call) and, for the last layer only, the value-row low half; what comes in is the first
+// layer's input and the weights.  Per accumulator element the MMAs, their order and the
+// epilogue's arithmetic are those of k_tc_gemm<FWD>, so the results are bitwise the same.
+// Measured against the per-layer launches (ms): 6x256 cavity at 69,632 points 0.480 -> 0.413,
+// loss only at 266,240 points 1.566 -> 1.127; 4x128 at 17,408 points 0.053 -> 0.027.  What
+// bounds it now: the MMAs, 219 cycles per K step where the tensor pipe alone would take 192
+// (the N = 64 ones read as much of A from shared memory as the others: 48 cycles instead of
+// 32), 8,000 of about 13,500 cycles per 256-wide layer and tile, then waits for weight stages.
+//
+// A layer is two jobs, each with one 256-column accumulator:
+//   M2 (a width above 128): the two 128-row m-tiles of one column tile, whose boxes are
+//      updated in place.  Both jobs take K chunks 0 and 1 (features 0-127) first, then both
+//      take chunks 2 and 3: the next layer's first half runs on what the first job's
+//      epilogue wrote while the second job's epilogue is still at work, and the first job's
+//      epilogue may overwrite chunks 0 and 1 once its own accumulator is complete.
+//   !M2 (widths <= 128): the same m-tile of two column tiles, one in each half of the
+//      boxes, so one tile's epilogue runs under the other tile's MMAs.
+//
+// Warp roles (384 threads): 0 weight producer, 1 TMEM allocator + MMA issuer, 2-9
+// epilogue, 10 input producer, 11 store issuer.  Barriers (all waits bounded, as in
+// k_tc_gemm; no role meets another at a named barrier):
+//   wfull/wempty[stage]  weight ring (hi and lo chunk of 128 rows x 64 K)
+//   afull[slot][chunk]   first-layer input chunk has landed
+//   afree[s]             the boxes of K half s (M2) or tile s (!M2) are free for new input
+//   accf[h]              job h's accumulator is complete, and the boxes its epilogue writes are read
+//   accr[h]              job h's epilogue has read its accumulator
+//   done[h]              job h's epilogue has written its boxes (every layer but the last)
+//   sread[h]             the bulk stores have read those boxes
+namespace {
+
+constexpr int FF_NT = FZ_NT + 32;
+constexpr int FF_CHUNK = 4 * FZ_BOX;              // 64 features x 256 columns: 32 KB
+constexpr int FF_HI = 4 * FF_CHUNK;               // 256 features of one tile, or 128 of two: 128 KB
+constexpr int FF_LO = 4 * FZ_BOX;                 // their value-row low halves: 32 KB
+constexpr int FF_WST = 2 * BM * 128;              // weight stage: W_hi and W_lo chunk, 32 KB
+constexpr int FF_WSTAGES = 2;
+constexpr size_t FF_SMEM = (size_t)FF_HI + FF_LO + (size_t)FF_WSTAGES * FF_WST + 1024 + 256;
+static_assert(FF_SMEM <= 227 * 1024, "fused forward: shared memory budget");
+
+struct FwdAllParams {
+  CUtensorMap in, in_lo;                     // first GEMM layer's input jets and low half
+  CUtensorMap w[PINN_MAX_HIDDEN], wlo[PINN_MAX_HIDDEN], out[PINN_MAX_HIDDEN];
+  int fin[PINN_MAX_HIDDEN], fout[PINN_MAX_HIDDEN];
+  const float* bias[PINN_MAX_HIDDEN];
+  __nv_bfloat16* a_last;                     // A_L, tile-major
+  __nv_bfloat16* alo_last;                   // its value-row low half
+  int layers, ntiles, reverse, jet_mode, wlo_values_only;
+  int store;                                 // write A_l of the layers below the last
+  int* status;
+  uint64_t wait_ns;
+};
+
+template <bool M2>
+__global__ void __launch_bounds__(FF_NT, 1) k_tc_fwd_all(const __grid_constant__ FwdAllParams p) {
+  constexpr int SLOTS = M2 ? 1 : 2;               // column tiles in flight
+  constexpr int SCH = M2 ? 4 : 2;                 // 64-feature chunks per slot
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  uint8_t* lob = smem + FF_HI;
+  uint8_t* wst = lob + FF_LO;
+  uint64_t* wfull = reinterpret_cast<uint64_t*>(wst + FF_WSTAGES * FF_WST);
+  uint64_t* wempty = wfull + FF_WSTAGES;
+  uint64_t* afull = wempty + FF_WSTAGES;          // [4]: slot * SCH + chunk
+  uint64_t* afree = afull + 4;                    // [2]
+  uint64_t* accf = afree + 2;                     // [2]
+  uint64_t* accr = accf + 2;                      // [2]
+  uint64_t* done = accr + 2;                      // [2]
+  uint64_t* sread = done + 2;                     // [2]
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(sread + 2);
+  volatile int* w_inflight = abort_flag + 1;      // [FF_WSTAGES]
+  volatile int* a_inflight = w_inflight + FF_WSTAGES;   // [4]
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(const_cast<int*>(a_inflight + 4));
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < FF_WSTAGES; ++i) {
+      mbar_init(&wfull[i], 1);
+      mbar_init(&wempty[i], 1);
+      w_inflight[i] = 0;
+    }
+    for (int i = 0; i < 4; ++i) { mbar_init(&afull[i], 1); a_inflight[i] = 0; }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&afree[i], p.store ? 2 : 1);      // the last layer's MMAs, and the store issuer
+      mbar_init(&accf[i], 1);
+      mbar_init(&accr[i], FZ_EPI);                // one arrival per epilogue warp
+      mbar_init(&done[i], FZ_EPI);
+      mbar_init(&sread[i], 1);
+    }
+    *abort_flag = 0;
+    fence_mbar_init();
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                 "r"(2 * BN));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+
+  const int g = (int)gridDim.x, L = p.layers;
+  // rounds of SLOTS tiles per CTA: tiles base, base + g, ...; job h of a round exists if its
+  // tile does (M2: both jobs work on the one tile)
+  auto has = [&](int base, int h) { return base + (M2 ? 0 : h * g) < p.ntiles; };
+  auto tile_of = [&](int base, int h) {
+    const int t = base + (M2 ? 0 : h) * g;
+    return p.reverse ? p.ntiles - 1 - t : t;
+  };
+  // whether job h of layer l has rows (an M2 layer of at most 128 rows has one m-tile)
+  auto rows = [&](int l, int h) { return !M2 || h == 0 || p.fout[l] > BM; };
+  // the K chunks of a layer in two halves (M2), or all at once
+  constexpr int HALVES = M2 ? 2 : 1, HCH = M2 ? 2 : 4;
+
+  if (warp == 0) {
+    // ---------------------------------------------------------------- weight producer
+    if (lane == 0) {
+      int st = 0;
+      uint32_t ph = 0;
+      bool ok = true;
+      for (int base = blockIdx.x; base < p.ntiles && ok; base += SLOTS * g)
+        for (int l = 0; l < L && ok; ++l) {
+          const int nk = (p.fin[l] + 63) >> 6;
+          for (int hh = 0; hh < 2 * HALVES && ok; ++hh) {
+            const int h = hh & 1, k0 = (hh >> 1) * HCH;
+            if (!has(base, h) || !rows(l, h)) continue;
+            for (int kb = k0; kb < min(nk, k0 + HCH); ++kb) {
+              if (!mbar_wait(&wempty[st], ph ^ 1, abort_flag, p.status, p.wait_ns)) { ok = false; break; }
+              uint8_t* sw = wst + st * FF_WST;
+              mbar_expect_tx(&wfull[st], FF_WST);
+              w_inflight[st] = (int)ph + 1;
+              tma_load_2d(sw, &p.w[l], &wfull[st], kb * 64, (M2 ? h : 0) * BM);
+              tma_load_2d(sw + BM * 128, &p.wlo[l], &wfull[st], kb * 64, (M2 ? h : 0) * BM);
+              if (++st == FF_WSTAGES) { st = 0; ph ^= 1; }
+            }
+          }
+        }
+    }
+  } else if (warp == 2 + FZ_EPI) {
+    // ---------------------------------------------------------------- input producer
+    if (lane == 0) {
+      const int nk = (p.fin[0] + 63) >> 6;
+      uint32_t round = 0;
+      bool ok = true;
+      for (int base = blockIdx.x; base < p.ntiles && ok; base += SLOTS * g, ++round) {
+        // one share of the boxes at a time: the K halves of the tile (M2), or the tiles
+        for (int s = 0; s < 2 && ok; ++s) {
+          if (!has(base, s)) continue;
+          if (round && !mbar_wait(&afree[s], (round - 1) & 1, abort_flag, p.status, p.wait_ns)) { ok = false; break; }
+          const int nb = tile_of(base, s), k0 = M2 ? HCH * s : 0;
+          for (int kb = k0; kb < min(nk, k0 + HCH); ++kb) {
+            const int c = (M2 ? 0 : s) * SCH + kb;
+            mbar_expect_tx(&afull[c], FF_CHUNK + FZ_BOX);
+            a_inflight[c] = (int)(round & 1) + 1;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) tma_load_3d(smem + c * FF_CHUNK + j * FZ_BOX, &p.in, &afull[c], j * 64, kb * 64, nb);
+            tma_load_3d(lob + c * FZ_BOX, &p.in_lo, &afull[c], 0, kb * 64, nb);
+          }
+        }
+        // the CTAs work in step, so their input loads come in bursts: the next round's input
+        // is brought into L2 under this round's layers
+        const int next = base + SLOTS * g;
+        for (int s = 0; s < SLOTS; ++s) {
+          if (next >= p.ntiles || !has(next, s)) break;
+          const int nb = tile_of(next, s);
+          for (int kb = 0; kb < nk; ++kb) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) tma_prefetch_3d(&p.in, j * 64, kb * 64, nb);
+            tma_prefetch_3d(&p.in_lo, 0, kb * 64, nb);
+          }
+        }
+      }
+    }
+  } else if (warp == 1) {
+    // ---------------------------------------------------------------- MMA issuer
+    if (lane == 0) {
+      constexpr uint32_t idesc = make_idesc(1u, 1u, BN), idesc64 = make_idesc(1u, 1u, TILE_PTS);
+      const uint32_t idesc_lo = p.wlo_values_only ? idesc64 : idesc;
+      int st = 0;
+      uint32_t ph = 0, round = 0;
+      int jobs[2] = {0, 0};                       // jobs issued per accumulator
+      int written[2] = {0, 0};                    // those of layers below the last
+      bool ok = true;
+      auto wait = [&](uint64_t* bar, uint32_t par) {
+        if (ok) ok = mbar_wait(bar, par, abort_flag, p.status, p.wait_ns);
+        return ok;
+      };
+      for (int base = blockIdx.x; base < p.ntiles && ok; base += SLOTS * g, ++round)
+        for (int l = 0; l < L && ok; ++l) {
+          const int nk = (p.fin[l] + 63) >> 6;
+          for (int hh = 0; hh < 2 * HALVES && ok; ++hh) {
+            const int h = hh & 1, half = hh >> 1, k0 = half * HCH;
+            if (!has(base, h)) continue;
+            const int slot = M2 ? 0 : h;
+            // this half's input boxes are written, and (first half) the accumulator is free
+            const int src = M2 ? half : h;
+            if (l > 0 && k0 < nk && (!M2 || h == 0) && !wait(&done[src], (uint32_t)(written[src] - 1) & 1)) break;
+            if (half == 0 && jobs[h] && !wait(&accr[h], (uint32_t)(jobs[h] - 1) & 1)) break;
+            tc_fence_after();
+            const uint32_t d = tmem_base + h * BN;
+            for (int kb = k0; kb < min(nk, k0 + HCH) && rows(l, h); ++kb) {
+              const int c = slot * SCH + kb;
+              if (l == 0) {
+                if (!wait(&afull[c], round & 1)) break;
+                a_inflight[c] = 0;
+              }
+              if (!wait(&wfull[st], ph)) break;
+              w_inflight[st] = 0;
+              tc_fence_after();
+              const uint32_t sa = smem_u32(wst + st * FF_WST), sa2 = sa + BM * 128;
+              const uint32_t sb = smem_u32(smem + c * FF_CHUNK), sl = smem_u32(lob + c * FZ_BOX);
+              // descriptors advance by 32 bytes (weights) and 16 rows of 128 bytes (jets) per K step,
+              // in units of 16 bytes
+              const uint64_t ad = make_desc(sa, 16, 1024), ad2 = make_desc(sa2, 16, 1024);
+              const uint64_t bd = make_desc(sb, FZ_BOX, 1024), bl = make_desc(sl, FZ_BOX, 1024);
+              const int left = p.fin[l] - 64 * kb;   // (K steps past it are zeros)
+#pragma unroll
+              for (int kk = 0; kk < 4; ++kk)
+                if (16 * kk < left) {
+                  tc_mma<false>(d, ad + 2 * kk, bd + 128 * kk, idesc, (kb > 0 || kk > 0) ? 1u : 0u);
+                  tc_mma<false>(d, ad2 + 2 * kk, bd + 128 * kk, idesc_lo, 1u);
+                  tc_mma<false>(d, ad + 2 * kk, bl + 128 * kk, idesc64, 1u);
+                }
+              tc_commit(&wempty[st]);
+              if (++st == FF_WSTAGES) { st = 0; ph ^= 1; }
+            }
+            if (!ok) break;
+            // M2: job 0 is complete after its second half; without one (K <= 128) only once
+            // job 1 has read the boxes too
+            if (!M2) {
+              tc_commit(&accf[h]);
+              if (l == L - 1) tc_commit(&afree[h]);
+            } else {
+              if (half == 1 && nk <= HCH && h == 1) tc_commit(&accf[0]);
+              if (half == 1 && (nk > HCH || h == 1)) tc_commit(&accf[h]);
+              if (l == L - 1 && h == 1) tc_commit(&afree[half]);   // both jobs are through with this half
+            }
+            if (half == HALVES - 1) {
+              ++jobs[h];
+              if (l < L - 1) ++written[h];
+            }
+          }
+        }
+    }
+  } else if (warp == 3 + FZ_EPI) {
+    // ---------------------------------------------------------------- store issuer
+    if (lane == 0 && p.store) {
+      int jobs[2] = {0, 0};
+      bool ok = true;
+      for (int base = blockIdx.x; base < p.ntiles && ok; base += SLOTS * g)
+        for (int l = 0; l < L && ok; ++l)
+          for (int h = 0; h < 2 && ok; ++h) {
+            if (!has(base, h)) continue;
+            if (l == L - 1) {   // no store reads these boxes any more
+              mbar_arrive(&afree[h]);
+              continue;
+            }
+            ok = mbar_wait(&done[h], (uint32_t)jobs[h] & 1, abort_flag, p.status, p.wait_ns);
+            if (!ok) break;
+            const int nb = tile_of(base, h);
+            for (int k = 0; k < 2 && rows(l, h); ++k) {
+              const int f = (M2 ? h : 0) * BM + 64 * k;
+              if (f >= p.fout[l]) break;
+              const uint8_t* src = smem + ((M2 ? 0 : h) * SCH + (M2 ? 2 * h : 0) + k) * FF_CHUNK;
+#pragma unroll
+              for (int r = 0; r < 4; ++r) tma_store_3d(&p.out[l], src + r * FZ_BOX, 64 * r, f, nb);
+            }
+            bulk_commit();
+            bulk_wait_read0();
+            mbar_arrive(&sread[h]);
+            ++jobs[h];
+          }
+      bulk_wait0();
+    }
+  } else {
+    // ---------------------------------------------------------------- epilogue
+    constexpr int UPTS = 16, UNITS = 2;
+    const int quad = warp & 3, part = (warp - 2) >> 2;
+    const int rr = quad * 32 + lane;                // accumulator row
+    int jobs[2] = {0, 0}, written[2] = {0, 0};
+    bool ok = true;
+    for (int base = blockIdx.x; base < p.ntiles && ok; base += SLOTS * g)
+      for (int l = 0; l < L && ok; ++l)
+        for (int h = 0; h < 2; ++h) {
+          if (!has(base, h)) continue;
+          const bool last = l == L - 1;
+          const int slot = M2 ? 0 : h, nb = tile_of(base, h), M = p.fout[l];
+          const int m = (M2 ? h : 0) * BM + rr;
+          const float bias = m < M ? p.bias[l][m] : 0.f;
+          ok = mbar_wait(&accf[h], (uint32_t)jobs[h] & 1, abort_flag, p.status, p.wait_ns);
+          if (__any_sync(0xffffffffu, !ok)) { ok = false; break; }   // (the warp's loads and shuffles are collective)
+          ++jobs[h];
+          tc_fence_after();
+          uint32_t hi[UNITS][4][8], lo[UNITS][8];   // packed BF16 results: 32 points x 4 rows, value-row low halves
+          if (rows(l, h)) {
+            const uint32_t tq = tmem_base + ((uint32_t)(quad * 32) << 16) + h * BN + part * (UNITS * UPTS);
+            const uint32_t keep = m < M ? 0xffffffffu : 0u;   // rows past the layer's width: zeros that pad the next K
+            auto unit = [&](int u, auto mode) {
+              float v[4][UPTS];
+#pragma unroll
+              for (int r = 0; r < 4; ++r) tmem_ld16_issue(tq + UPTS * u + 64 * r, v[r]);
+              tmem_wait_ld();
+              if (u == UNITS - 1) {
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&accr[h]);
+              }
+              fwd_pairs<decltype(mode)::value>(v, bias, hi[u], lo[u], keep);
+            };
+            auto units = [&](auto mode) {
+#pragma unroll
+              for (int u = 0; u < UNITS; ++u) unit(u, mode);
+            };
+            if (p.jet_mode == JET_NS) units(std::integral_constant<int, JET_NS>{});
+            else if (p.jet_mode == JET_BURGERS) units(std::integral_constant<int, JET_BURGERS>{});
+            else units(std::integral_constant<int, JET_MAXWELL>{});
+          } else if (lane == 0) {
+            mbar_arrive(&accr[h]);
+          }
+          if (last) {
+            if (rows(l, h) && m < M) {
+              const int pc = part * (UNITS * UPTS);
+              __nv_bfloat16* ao = p.a_last + toff(m, (int64_t)nb * BN, M) + pc;
+              __nv_bfloat16* al = p.alo_last + loff(m, (int64_t)nb * TILE_PTS, M) + pc;
+#pragma unroll
+              for (int u = 0; u < UNITS; ++u) {
+#pragma unroll
+                for (int r = 0; r < 4; ++r) st_global_256(ao + UPTS * u + 64 * r, hi[u][r]);
+                st_global_256(al + UPTS * u, lo[u]);
+              }
+            }
+            continue;
+          }
+          // the bulk stores of these boxes' previous contents have read them
+          if (p.store && written[h]) {
+            ok = mbar_wait(&sread[h], (uint32_t)(written[h] - 1) & 1, abort_flag, p.status, p.wait_ns);
+            if (__any_sync(0xffffffffu, !ok)) { ok = false; break; }
+          }
+          ++written[h];
+          if (rows(l, h)) {
+            const int c = slot * SCH + (M2 ? 2 * h : 0) + (rr >> 6);
+            const uint32_t row = smem_u32(smem + c * FF_CHUNK + (rr & 63) * 128);
+            const uint32_t lrow = smem_u32(lob + c * FZ_BOX + (rr & 63) * 128);
+#pragma unroll
+            for (int u = 0; u < UNITS; ++u)
+#pragma unroll
+              for (int q = 0; q < 2; ++q) {
+                const uint32_t at = (uint32_t)(((part * 4 + 2 * u + q) ^ (rr & 7)) << 4);
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+                  asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(row + r * FZ_BOX + at), "r"(hi[u][r][4 * q]),
+                               "r"(hi[u][r][4 * q + 1]), "r"(hi[u][r][4 * q + 2]), "r"(hi[u][r][4 * q + 3])
+                               : "memory");
+                asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(lrow + at), "r"(lo[u][4 * q]),
+                             "r"(lo[u][4 * q + 1]), "r"(lo[u][4 * q + 2]), "r"(lo[u][4 * q + 3])
+                             : "memory");
+              }
+            fence_proxy_async_smem();               // these writes before the MMAs' and bulk stores' reads
+          }
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&done[h]);
+        }
+  }
+
+  // ---- teardown: wait (bounded) for copies still in flight, free TMEM ----------------
+  __syncthreads();
+  if (threadIdx.x == 0 && *abort_flag) {
+    auto drain = [&](uint64_t* bar, int f) {
+      if (!f) return;
+      const uint64_t t0 = gtimer();
+      while (!mbar_try(bar, (uint32_t)(f - 1)) && gtimer() - t0 < WAIT_NS) {}
+    };
+    for (int i = 0; i < FF_WSTAGES; ++i) drain(&wfull[i], w_inflight[i]);
+    for (int i = 0; i < 4; ++i) drain(&afull[i], a_inflight[i]);
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(2 * BN));
+  }
+}
+
+}  // namespace
+
+bool tc_fwd_all_supported(const pinn_handle* h, int64_t NC) {
+  if (h->spec.precision != PINN_BF16 || h->act != PINN_ACT_TANH || h->first_gemm >= h->L) return false;
+  for (int li = h->first_gemm; li < h->L; ++li)
+    if (!tc_layer_supported(h, li, NC) || h->layers[li].fin > 256 || h->layers[li].fout > 256) return false;
+  return true;
+}
+
+pinn_status tc_gemm_fwd_all(pinn_handle* h, const TcFwdLayer* layers, int n, const void* in, const void* in_lo,
+                            void* alo_last, int64_t NC, int jet_mode, int reverse, int store, cudaStream_t st) {
+  FwdAllParams p;
+  const uint64_t nt = (uint64_t)(NC / TILE_COLS);
+  bool ok = make_map3(&p.in, in, false, TILE_COLS, layers[0].fin, nt, 64, 64) &&
+            make_map3(&p.in_lo, in_lo, false, TILE_PTS, layers[0].fin, nt, 64, 64);
+  bool m2 = false;
+  for (int l = 0; l < n && ok; ++l) {
+    const TcFwdLayer& y = layers[l];
+    ok = make_map(&p.w[l], y.W, false, y.fin, y.fout, 64, BM) && make_map(&p.wlo[l], y.Wlo, false, y.fin, y.fout, 64, BM) &&
+         make_map3(&p.out[l], y.out, false, TILE_COLS, y.fout, nt, 64, 64);
+    p.fin[l] = y.fin; p.fout[l] = y.fout; p.bias[l] = y.bias;
+    m2 = m2 || y.fin > BM || y.fout > BM;
+  }
+  if (!ok) return map_err(h, "fused forward");
+  p.a_last = reinterpret_cast<__nv_bfloat16*>(layers[n - 1].out);
+  p.alo_last = reinterpret_cast<__nv_bfloat16*>(alo_last);
+  p.layers = n; p.ntiles = (int)nt; p.reverse = reverse; p.jet_mode = jet_mode;
+  p.store = store && n > 1;   // (a single layer leaves through the epilogue)
+  p.wlo_values_only = (h->spec.flags & PINN_FLAG_BF16_VALUE_SPLIT) ? 1 : 0;
+  p.status = h->d_status;
+  p.wait_ns = WAIT_NS;
+  static bool attr_set[2] = {false, false};
+  auto kern = m2 ? k_tc_fwd_all<true> : k_tc_fwd_all<false>;
+  const pinn_status s = reserve_smem(h, kern, FF_SMEM, attr_set[m2 ? 1 : 0], "fused forward kernel");
+  if (s) return s;
+  kern<<<grid_for(h, p.ntiles), FF_NT, FF_SMEM, st>>>(p);
+  return launch_check(h, "fused forward");
+}
 
 TcBatch* tc_batch_create() { return new (std::nothrow) TcBatch(); }
 

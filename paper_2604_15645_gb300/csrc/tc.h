@@ -30,6 +30,17 @@ int tc_dw_splits(const pinn_handle* h, int fout, int fin, int64_t NC);
 //         the epilogue also writes e.out_pm (point-major A_l) when set.
 pinn_status tc_gemm_fwd(pinn_handle* h, const void* W, const void* Wlo, const void* A, const void* Alo, int fout,
                         int fin, int64_t NC, const EpiArgs& e, cudaStream_t st);
+// Every hidden GEMM layer of the forward in one launch (BF16 tanh networks whose hidden
+// widths and first fan-in are at most 256), bitwise the per-layer launches.  `in` / `in_lo`
+// are the first layer's input jets and low half; each layer's out receives A_l (with
+// store = 0, a loss-only call, only the last layer's does), alo_last the low half of A_L.
+struct TcFwdLayer {
+  const void* W; const void* Wlo; const float* bias; void* out;
+  int fin, fout;
+};
+bool tc_fwd_all_supported(const pinn_handle* h, int64_t NC);
+pinn_status tc_gemm_fwd_all(pinn_handle* h, const TcFwdLayer* layers, int n, const void* in, const void* in_lo,
+                            void* alo_last, int64_t NC, int jet_mode, int reverse, int store, cudaStream_t st);
 // Abar = W^T Zbar (tanh-jet adjoint epilogue), WT [fin][fout].
 //   BF16: Zbar^T [fout][NC] tile-major, high halves only (WTlo unused).
 //   TF32: (WT_hi + WT_lo) Zbar + WT_hi (Zbar - tf32(Zbar)), Zbar point-major [NC][fout];

@@ -67,3 +67,41 @@ def test_causal_segment_sums(cuda_lib, precision, width, segments, n_res):
     assert abs(t[1] - terms["pde"]) <= tol * abs(terms["pde"])
     assert np.linalg.norm(g.cpu().numpy() - rg) <= tol * np.linalg.norm(rg)
     assert np.allclose(net.causal_weights().cpu().numpy(), terms["causal_weights"], rtol=10 * tol)
+
+
+@pytest.mark.parametrize("widths,ff", [
+    ([16, 16], 0),                    # one GEMM layer, a quarter of a K chunk
+    ([128, 72, 128], 64),             # at most 128 wide: two column tiles in flight
+    ([136, 24, 256, 16, 200], 8),     # m-tiles of 136 and 200 rows, layers with one m-tile in between
+    ([256, 256], 128),                # full 256
+])
+@pytest.mark.parametrize("n_res", [1, 20000])   # one tile, and more tiles than two rounds of every SM
+def test_fused_forward_edges(cuda_lib, widths, ff, n_res):
+    """The one-kernel forward gives bitwise the losses and gradients of the per-layer
+    launches (which the grouped many-network step runs; those are checked against the
+    oracle elsewhere), and a loss-only call gives the same loss."""
+    from paper_2604_15645_gb300 import api
+    spec = NetSpec(PDE_BURGERS, 2, 1, widths, ff_m=ff, ff_sigma=1.0, rwf=True)
+    p, B = init_params(spec, 91, 0.2), ff_matrix(spec, 92)
+    b = make_batch(PDE_BURGERS, n_res, 30, 20, 93, 94)
+    prob, db = api.make_problem(0.02), api.DeviceBatch.from_host(b)
+    params = torch.tensor(p, device="cuda")
+    Bd = None if B is None else torch.tensor(B, device="cuda")
+    res = []
+    for grouped in (False, True):
+        multi = api.PinnMulti([spec], "bf16")
+        if Bd is not None:
+            api._lib.check_multi(api._lib.load().pinn_multi_set_ff_matrix(multi.h, 0, Bd.data_ptr()), multi.h)
+        multi.set_inputs([db], [prob])
+        multi.grouped = grouped
+        q = params.clone()
+        grad, m, v = (torch.zeros_like(q) for _ in range(3))
+        loss = multi.train_step(q, grad, m, v, step=1)
+        torch.cuda.synchronize()
+        assert multi.status_poll() == 0
+        res.append((loss[0].clone(), grad))
+    assert torch.equal(res[0][0], res[1][0]) and torch.equal(res[0][1], res[1][1])
+    net = api.PinnNet.from_spec(spec, "bf16")
+    if Bd is not None:
+        net.set_ff_matrix(B)
+    assert torch.equal(net.loss(params, db, prob), res[0][0])
