@@ -133,6 +133,28 @@ __device__ __forceinline__ void jet_adj_a(const float a[4], const float ab[4], f
   }
 }
 
+// jet_adj_a of two points at once in packed FP32, with the scalar rule's roundings.
+template <int MODE>
+__device__ __forceinline__ void jet_adj_a2(const f32x2 a[4], const f32x2 ab[4], f32x2 zb[4]) {
+  const f32x2 one = dup2(1.f), t = a[0];
+  const f32x2 tp = mul2(fma2(t, dup2(-1.f), one), add2(one, t));
+  zb[3] = mul2(ab[3], tp);
+  if (MODE == JET_MAXWELL) {
+    zb[1] = mul2(ab[1], tp);
+    zb[2] = mul2(ab[2], tp);
+    const f32x2 x = fma2(ab[3], a[3], fma2(ab[1], a[1], mul2(ab[2], a[2])));
+    zb[0] = fma2(ab[0], tp, mul2(mul2(t, dup2(-2.f)), x));
+  } else {
+    const f32x2 q = (MODE == JET_NS) ? fma2(a[1], a[1], mul2(a[2], a[2])) : mul2(a[1], a[1]);
+    const f32x2 m4 = mul2(mul2(ab[3], dup2(-4.f)), t);
+    zb[1] = fma2(ab[1], tp, mul2(m4, a[1]));
+    zb[2] = (MODE == JET_NS) ? fma2(ab[2], tp, mul2(m4, a[2])) : mul2(ab[2], tp);
+    const f32x2 x = fma2(ab[1], a[1], mul2(ab[2], a[2]));
+    const f32x2 y = fma2(t, x, mul2(ab[3], fma2(t, a[3], q)));
+    zb[0] = fma2(ab[0], tp, mul2(y, dup2(-2.f)));
+  }
+}
+
 // ---- periodic activation sin(omega z) ----------------------------------------------
 // The sine activation (periodic activation function, Sec. 2.6) uses the same jet rule
 // with t = sin(w z), t' = w cos(w z), t'' = -w^2 sin(w z), t''' = -w^3 cos(w z).  Its
