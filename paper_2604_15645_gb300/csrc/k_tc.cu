@@ -203,6 +203,44 @@ __device__ __forceinline__ void adj_pairs8(float (&v)[4][N], int first, const ui
   }
 }
 
+// A lane of an epilogue warp holds a feature's 32 points of a jet row as two 32-byte sectors
+// (a: points 0-15, b: 16-31).  After the swap within lane pairs, one access of the even
+// lane and one of the odd lane cover 64 consecutive bytes: a and b are the sectors
+// 16 (lane & 1) of the pair's even and of its odd feature.  (Its own inverse: loads swap back.)
+// Every 128-byte line that an instruction touches takes a cycle of the data path that shared
+// memory, the MMAs' operand reads and the bulk copies share, and that path bounds the wide
+// kernels: 16 lines per instruction instead of 32.
+__device__ __forceinline__ void pair_swap(uint32_t (&a)[8], uint32_t (&b)[8]) {
+  const bool odd = threadIdx.x & 1;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const uint32_t y = __shfl_xor_sync(0xffffffffu, odd ? a[i] : b[i], 1);
+    const uint32_t keep_a = a[i];
+    a[i] = odd ? y : keep_a;
+    b[i] = odd ? b[i] : y;
+  }
+}
+// Stores 32 points x 4 rows of a warp's features (w[unit][row], BF16 pairs): column pc of tile
+// nb, feature m of M (M even, so a pair of lanes is valid together).
+__device__ __forceinline__ void store_pairs(__nv_bfloat16* out, uint32_t (&w)[2][4][8], int m, int64_t nb, int M, int pc) {
+  __nv_bfloat16* o = out + toff(m & ~1, nb * BN, M) + pc + 16 * (m & 1);
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    pair_swap(w[0][r], w[1][r]);
+    if (m < M) {
+      st_global_256(o + 64 * r, w[0][r]);
+      st_global_256(o + 64 * r + TILE_COLS, w[1][r]);
+    }
+  }
+}
+__device__ __forceinline__ void store_lo_pairs(__nv_bfloat16* out, uint32_t (&w)[2][8], int m, int64_t nb, int M, int pc) {
+  __nv_bfloat16* o = out + loff(m & ~1, nb * TILE_PTS, M) + pc + 16 * (m & 1);
+  pair_swap(w[0], w[1]);
+  if (m < M) {
+    st_global_256(o, w[0]);
+    st_global_256(o + TILE_PTS, w[1]);
+  }
+}
 // Calls f with the jet rule as a compile-time constant.
 template <typename F>
 __device__ __forceinline__ void with_jet_mode(int mode, F&& f) {
@@ -493,6 +531,9 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA, const CUte
     const int row = quad * 32 + lane;
     auto unit_col = [&](int u) { return part * (UNITS * UPTS) + UPTS * u; };
 
+    // BF16 tanh forward: both units of a warp's tile are finished before their sectors are exchanged
+    // and stored; the accumulator is free as soon as it is in registers.
+    constexpr bool PAIRS = !TF32 && !SINE && MODE == TC_FWD;
     constexpr int ZR = 4;                                // jet rows loaded per unit
     uint32_t znext[ZR][ZW];                              // adjoint: A rows of the next unit
     auto load_z = [&](int t_, int u_) {
@@ -511,7 +552,6 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA, const CUte
     if constexpr (MODE == TC_ADJ && !SINE) {
       if (grid.bx() < total) load_z(grid.bx(), 0);
     }
-
     int local = 0;
     for (int t = grid.bx(); t < total; t += grid.gdim(), ++local) {
       int mb, nb, k0, k1;
@@ -648,7 +688,24 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA, const CUte
         }
       };
 
-      if constexpr (PIPE) {
+      if constexpr (PAIRS) {
+        uint32_t w[UNITS][4][8], lo[UNITS][8];
+        const float bias = mvalid ? p.e.bias[m] : 0.f;
+#pragma unroll
+        for (int u = 0; u < UNITS; ++u) {
+          float v[4][UPTS];
+          issue(u, v);
+          tmem_wait_ld();
+          if (u == UNITS - 1) {
+            tc_fence_before();
+            mbar_arrive(&acc_empty[buf]);
+          }
+          with_jet_mode(p.e.jet_mode,
+                        [&](auto mode) { fwd_pairs<decltype(mode)::value>(v, bias, w[u], lo[u], 0xffffffffu); });
+        }
+        store_pairs(reinterpret_cast<T*>(p.e.out), w, m, nb, p.M, unit_col(0));
+        if (p.e.alo_out) store_lo_pairs(reinterpret_cast<T*>(p.e.alo_out), lo, m, nb, p.M, unit_col(0));
+      } else if constexpr (PIPE) {
         float va[4][UPTS], vb[4][UPTS];
         issue(0, va);
         tmem_wait_ld();
@@ -678,8 +735,10 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA, const CUte
           if (j < p.e.dterms) dst[1 + j] = db[1 + j];
       }
       }   // half
-      tc_fence_before();
-      mbar_arrive(&acc_empty[buf]);
+      if constexpr (!PAIRS) {
+        tc_fence_before();
+        mbar_arrive(&acc_empty[buf]);
+      }
     }
   }
 
@@ -799,8 +858,6 @@ pinn_status launch_group(pinn_handle* h, const TcGroupEntry* d_tab, int n, int b
   kern<<<blocks, C::NTHREADS, C::SMEM, st>>>(d_tab, n);
   return launch_check(h, "grouped tcgen05 kernel");
 }
-
-pinn_status launch_adjdw_group(pinn_handle* h, const TcGroupEntry* d_tab, int n, int blocks, cudaStream_t st);
 
 }  // namespace
 
@@ -944,12 +1001,16 @@ pinn_status fwd_impl(pinn_handle* h, const void* W, const void* Wlo, const void*
   return launch<TF32, TC_FWD, true>(h, ma, ma2, mb, mlo, p, grid, st);
 }
 
+pinn_status adj_staged(pinn_handle* h, const void* WT, const void* Zbar, int fin, int fout, int64_t NC,
+                       const EpiArgs& e, cudaStream_t st);
+
 template <bool TF32>
 pinn_status adj_impl(pinn_handle* h, const void* WT, const void* WTlo, const void* Zbar, int fin, int fout,
                      int64_t NC, const EpiArgs& e, cudaStream_t st) {
   // TF32: split weights and the point-major adjoint with its low half (three MMAs);
   // BF16: high halves only.
   constexpr bool SPLIT = TF32;
+  if (!TF32 && h->act != PINN_ACT_SINE) return adj_staged(h, WT, Zbar, fin, fout, NC, e, st);
   using C = Cfg<TF32, TC_ADJ, SPLIT>;
   CUtensorMap ma, ma2, mb;
   if (!make_map(&ma, WT, TF32, fout, fin, C::BKE, BM)) return map_err(h, "adjoint weights");
@@ -964,9 +1025,7 @@ pinn_status adj_impl(pinn_handle* h, const void* WT, const void* WTlo, const voi
   TcParams p = base_params(fin, (int)NC, fout, NC, C::BKE, h->d_status);
   p.e = e;
   const int grid = grid_for(h, p.m_tiles * p.n_tiles);
-  if constexpr (!TF32)
-    if (h->act == PINN_ACT_SINE) return launch<TF32, TC_ADJ, SPLIT, true>(h, ma, ma2, mb, mb, p, grid, st);
-  return launch<TF32, TC_ADJ, SPLIT>(h, ma, ma2, mb, mb, p, grid, st);
+  return launch<TF32, TC_ADJ, SPLIT, !TF32>(h, ma, ma2, mb, mb, p, grid, st);
 }
 
 template <bool TF32>
@@ -1036,8 +1095,15 @@ pinn_status tc_gemm_dw(pinn_handle* h, const void* Zbar, const void* A, int fout
 // now: the path of shared memory, which the MMAs' operands (N = 64: 6 KB per 32 cycles),
 // the bulk copies and the stores share.
 //
+// DW = false is the adjoint alone, for a layer whose fan-out is above 256 (its dW^T slab
+// would fill tensor memory).  Two accumulators overlap the epilogue with the next unit's MMAs;
+// the epilogue puts Zbar_{l-1} in the place of the staged activations and the tile leaves by
+// bulk tensor stores, so no lane stores (or loads) 32-byte sectors of 32 different lines:
+// 8x512 cavity at 1,064,960 points, seven launches 18.5 -> 16.5 ms, Maxwell 5x512 at 294,912,
+// four 3.04 -> 2.56 ms.  (With DW = true the in-place stores were slower, 0.471 -> 0.479 ms.)
+//
 // Warp roles (352 threads): 0 stage producer (W^T chunk + Zbar chunk), 1 TMEM
-// allocator + MMA issuer, 2-9 epilogue, 10 A-tile producer.
+// allocator + MMA issuer, 2-9 epilogue, 10 A tiles in, Zbar tiles out.
 namespace {
 
 constexpr int FZ_EPI = EPI_WARPS;
@@ -1046,18 +1112,22 @@ constexpr int FZ_WB = BM * 128;                  // W^T chunk [128 fin][64 fout]
 constexpr int FZ_BOX = 64 * 128;                 // Zbar box [64 fout][64 cols]         8 KB
 constexpr int FZ_ZB = 4 * FZ_BOX;                // Zbar chunk [64 fout][256 cols]     32 KB
 constexpr int FZ_STAGE = FZ_WB + FZ_ZB;          // 48 KB
-constexpr int FZ_STAGES = 2;
 constexpr int FZ_ABOX = BM * 128;                // A box [128 fin][64 cols]           16 KB
 constexpr int FZ_AT = 4 * FZ_ABOX;               // A_{l-1} tile [128 fin][256 cols]   64 KB
-constexpr int FZ_ABUF = 2;
-constexpr size_t FZ_SMEM = (size_t)FZ_STAGES * FZ_STAGE + (size_t)FZ_ABUF * FZ_AT + 1024 + 256;
-static_assert(FZ_SMEM <= 227 * 1024, "fused adjoint: shared memory budget");
 constexpr int FZ_DW_COL = BN;                    // dW^T accumulator: TMEM columns 256..511
+template <bool DW>
+struct FzCfg {
+  static constexpr int STAGES = DW ? 2 : 3;
+  static constexpr int ABUF = DW ? 2 : 1;
+  static constexpr size_t SMEM = (size_t)STAGES * FZ_STAGE + (size_t)ABUF * FZ_AT + 1024 + 256;
+  static_assert(SMEM <= 227 * 1024, "fused adjoint: shared memory budget");
+};
 
-template <typename Grid>
-__device__ __forceinline__ void tc_adjdw_body(const CUtensorMap* mapW, const CUtensorMap* mapZ,
-                                              const CUtensorMap* mapA, const TcParams& p, const Grid grid) {
-  using T = __nv_bfloat16;
+template <bool DW, typename Grid>
+__device__ __forceinline__ void tc_adjdw_body(const CUtensorMap* mapW, const CUtensorMap* mapZ, const CUtensorMap* mapA,
+                                              const CUtensorMap* mapO, const TcParams& p, const Grid grid) {
+  constexpr int FZ_STAGES = FzCfg<DW>::STAGES, FZ_ABUF = FzCfg<DW>::ABUF;
+  constexpr int ACC = DW ? 1 : 2;                // adjoint accumulators
   extern __shared__ uint8_t smem_raw[];
   // 1024-byte aligned by offsetting the shared array itself (an integer round trip would
   // hide the address space and turn every shared access below into a generic one)
@@ -1066,10 +1136,10 @@ __device__ __forceinline__ void tc_adjdw_body(const CUtensorMap* mapW, const CUt
   uint64_t* full = reinterpret_cast<uint64_t*>(abase + FZ_ABUF * FZ_AT);
   uint64_t* empty = full + FZ_STAGES;
   uint64_t* acc_full = empty + FZ_STAGES;
-  uint64_t* acc_empty = acc_full + 1;
-  uint64_t* a_full = acc_empty + 1;
-  uint64_t* a_empty = a_full + FZ_ABUF;
-  uint64_t* dw_full = a_empty + FZ_ABUF;
+  uint64_t* acc_empty = acc_full + ACC;
+  uint64_t* a_full = acc_empty + ACC;
+  uint64_t* z_done = a_full + FZ_ABUF;
+  uint64_t* dw_full = z_done + FZ_ABUF;
   volatile int* abort_flag = reinterpret_cast<volatile int*>(dw_full + 1);
   volatile int* inflight = abort_flag + 1;              // [FZ_STAGES]
   volatile int* a_inflight = inflight + FZ_STAGES;      // [FZ_ABUF]
@@ -1084,11 +1154,13 @@ __device__ __forceinline__ void tc_adjdw_body(const CUtensorMap* mapW, const CUt
     }
     for (int b = 0; b < FZ_ABUF; ++b) {
       mbar_init(&a_full[b], 1);
-      mbar_init(&a_empty[b], 1 + 32 * FZ_EPI);   // the dW MMAs' commit + every epilogue thread
+      mbar_init(&z_done[b], FZ_EPI);   // one arrival per epilogue warp
       a_inflight[b] = 0;
     }
-    mbar_init(acc_full, 1);
-    mbar_init(acc_empty, 32 * FZ_EPI);
+    for (int b = 0; b < ACC; ++b) {
+      mbar_init(&acc_full[b], 1);
+      mbar_init(&acc_empty[b], FZ_EPI);
+    }
     mbar_init(dw_full, 1);
     *abort_flag = 0;
     fence_mbar_init();
@@ -1141,20 +1213,51 @@ __device__ __forceinline__ void tc_adjdw_body(const CUtensorMap* mapW, const CUt
       }
     }
   } else if (warp == 2 + FZ_EPI) {
-    // ---------------------------------------------------------------- A-tile producer
+    // ---------------------------------------------------------------- A tiles in (and Zbar tiles out)
     if (lane == 0) {
-      int local = 0;
-      for (int t = grid.bx(); t < total && !*abort_flag; t += grid.gdim(), ++local) {
+      int in = 0, out = 0;    // tiles loaded, tiles done by the epilogue
+      int t_out = grid.bx();
+      bool ok = true;
+      // the next tile is done; staged: it leaves by bulk tensor stores
+      auto next_done = [&]() {
+        const int ab = out % FZ_ABUF;
+        ok = mbar_wait(&z_done[ab], (uint32_t)(out / FZ_ABUF) & 1, abort_flag, p.status, p.wait_ns);
+        if (!ok) return;
+        if constexpr (!DW) {
+          int mb, nb;
+          coords(t_out, mb, nb);
+          const uint8_t* at = abase + ab * FZ_AT;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) tma_store_3d(mapO, at + j * FZ_ABOX, j * 64, mb * BM, nb);
+          bulk_commit();
+        }
+        t_out += grid.gdim();
+        ++out;
+      };
+      for (int t = grid.bx(); t < total && ok && !*abort_flag; t += grid.gdim(), ++in) {
         int mb, nb;
         coords(t, mb, nb);
-        const int ab = local & 1;
-        const uint32_t aph = (uint32_t)(local >> 1) & 1;
-        if (!mbar_wait(&a_empty[ab], aph ^ 1, abort_flag, p.status, p.wait_ns)) break;
+        const int ab = in % FZ_ABUF;
+        if (in >= FZ_ABUF) {
+          next_done();
+          if (!ok) break;
+          if (!DW) bulk_wait_read0();
+        }
         mbar_expect_tx(&a_full[ab], FZ_AT);
-        a_inflight[ab] = (int)aph + 1;
+        a_inflight[ab] = ((in / FZ_ABUF) & 1) + 1;
         uint8_t* at = abase + ab * FZ_AT;
 #pragma unroll
         for (int j = 0; j < 4; ++j) tma_load_3d(at + j * FZ_ABOX, mapA, &a_full[ab], j * 64, mb * BM, nb);
+        if (!DW && t + grid.gdim() < total) {   // one buffer: the next tile waits in L2
+          int mn, nn;
+          coords(t + grid.gdim(), mn, nn);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) tma_prefetch_3d(mapA, j * 64, mn * BM, nn);
+        }
+      }
+      if constexpr (!DW) {
+        while (ok && out < in && !*abort_flag) next_done();
+        bulk_wait0();
       }
     }
   } else if (warp == 1) {
@@ -1162,17 +1265,18 @@ __device__ __forceinline__ void tc_adjdw_body(const CUtensorMap* mapW, const CUt
     if (lane == 0) {
       constexpr uint32_t idesc_adj = make_idesc(1u, 1u, BN);   // W^T . Zbar, B MN-major, N = 256
       constexpr uint32_t idesc_dw = make_idesc(1u, 0u, 64);    // A_{l-1} . Zbar chunk^T, both K-major, N = 64
-      const uint32_t d_adj = tmem_base;
       const uint32_t d_dw = tmem_base + FZ_DW_COL;
       int stage = 0;
       uint32_t phase = 0;
       int local = 0;
       bool ok = true;
       for (int t = grid.bx(); t < total && !*abort_flag && ok; t += grid.gdim(), ++local) {
-        const int ab = local & 1;
-        if (!mbar_wait(&a_full[ab], (uint32_t)(local >> 1) & 1, abort_flag, p.status, p.wait_ns)) { ok = false; break; }
-        a_inflight[ab] = 0;
-        tc_fence_after();
+        const int ab = local % FZ_ABUF, buf = local % ACC;
+        const uint32_t d_adj = tmem_base + buf * BN;
+        if constexpr (DW) {
+          if (!mbar_wait(&a_full[ab], (uint32_t)(local / FZ_ABUF) & 1, abort_flag, p.status, p.wait_ns)) { ok = false; break; }
+          tc_fence_after();
+        }
         const uint32_t sa_t = smem_u32(abase + ab * FZ_AT);
         for (int kb = 0; kb < p.k_iters; ++kb) {
           if (!mbar_wait(&full[stage], phase, abort_flag, p.status, p.wait_ns)) { ok = false; break; }
@@ -1181,16 +1285,18 @@ __device__ __forceinline__ void tc_adjdw_body(const CUtensorMap* mapW, const CUt
           const uint32_t sw = smem_u32(smem + stage * FZ_STAGE);
           const uint32_t sz = sw + FZ_WB;
           // weight gradient of this 64-row fout chunk: dW^T[:, 64 kb ..] += A_tile . Zbar_chunk^T
+          if constexpr (DW) {
 #pragma unroll
-          for (int j = 0; j < 4; ++j)
+            for (int j = 0; j < 4; ++j)
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk)
-              tc_mma<false>(d_dw + 64 * kb, make_desc(sa_t + j * FZ_ABOX + kk * 32, 16, 1024),
-                            make_desc(sz + j * FZ_BOX + kk * 32, 16, 1024), idesc_dw,
-                            (local > 0 || j > 0 || kk > 0) ? 1u : 0u);
+              for (int kk = 0; kk < 4; ++kk)
+                tc_mma<false>(d_dw + 64 * kb, make_desc(sa_t + j * FZ_ABOX + kk * 32, 16, 1024),
+                              make_desc(sz + j * FZ_BOX + kk * 32, 16, 1024), idesc_dw,
+                              (local > 0 || j > 0 || kk > 0) ? 1u : 0u);
+          }
           if (kb == 0) {
-            // the single adjoint accumulator: wait until the epilogue has copied out the last tile
-            if (!mbar_wait(acc_empty, ((uint32_t)local & 1) ^ 1, abort_flag, p.status, p.wait_ns)) { ok = false; break; }
+            // wait until the epilogue has copied out the accumulator's last tile
+            if (!mbar_wait(&acc_empty[buf], ((uint32_t)(local / ACC) & 1) ^ 1, abort_flag, p.status, p.wait_ns)) { ok = false; break; }
             tc_fence_after();
           }
 #pragma unroll
@@ -1201,10 +1307,9 @@ __device__ __forceinline__ void tc_adjdw_body(const CUtensorMap* mapW, const CUt
           if (++stage == FZ_STAGES) { stage = 0; phase ^= 1; }
         }
         if (!ok) break;
-        tc_commit(&a_empty[ab]);
-        tc_commit(acc_full);
+        tc_commit(&acc_full[buf]);
       }
-      if (ok && !*abort_flag) tc_commit(dw_full);
+      if (DW && ok && !*abort_flag) tc_commit(dw_full);
     }
   } else {
     // ---------------------------------------------------------------- epilogue
@@ -1224,19 +1329,23 @@ __device__ __forceinline__ void tc_adjdw_body(const CUtensorMap* mapW, const CUt
       mb_cta = mb;
       float xc[3] = {0.f, 0.f, 0.f};
       if (p.e.dbpart && p.e.dterms) lane_coords(p.e, (int64_t)nb * TILE_PTS + part * 32 + lane, xc);
-      if (!mbar_wait(acc_full, (uint32_t)local & 1, abort_flag, p.status, p.wait_ns)) break;
+      const int ab = local % FZ_ABUF, buf = local % ACC;
+      bool ok = mbar_wait(&acc_full[buf], (uint32_t)(local / ACC) & 1, abort_flag, p.status, p.wait_ns);
+      if (__any_sync(0xffffffffu, !ok)) break;   // (the warp's loads and shuffles are collective)
       tc_fence_after();
       float v[UNITS][4][UPTS];
 #pragma unroll
       for (int u = 0; u < UNITS; ++u)
 #pragma unroll
-        for (int r = 0; r < 4; ++r) tmem_ld16_issue(tq + unit_col(u) + 64 * r, v[u][r]);
+        for (int r = 0; r < 4; ++r) tmem_ld16_issue(tq + buf * BN + unit_col(u) + 64 * r, v[u][r]);
       tmem_wait_ld();
       tc_fence_before();
-      mbar_arrive(acc_empty);            // the next tile's adjoint MMAs may overwrite it now
-      const int ab = local & 1;
-      if (!mbar_wait(&a_full[ab], (uint32_t)(local >> 1) & 1, abort_flag, p.status, p.wait_ns)) break;
-      const uint8_t* at = abase + ab * FZ_AT;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&acc_empty[buf]);   // the next tile's adjoint MMAs may overwrite it now
+      ok = mbar_wait(&a_full[ab], (uint32_t)(local / FZ_ABUF) & 1, abort_flag, p.status, p.wait_ns);
+      if (__any_sync(0xffffffffu, !ok)) break;
+      a_inflight[ab] = 0;
+      uint8_t* at = abase + ab * FZ_AT;
       const int m = mb * BM + rr;
       const bool mvalid = m < p.M;
       float db[4] = {0.f, 0.f, 0.f, 0.f};
@@ -1245,22 +1354,38 @@ __device__ __forceinline__ void tc_adjdw_body(const CUtensorMap* mapW, const CUt
         const int pc = unit_col(u);
 #pragma unroll
         for (int h8 = 0; h8 < UPTS / 8; ++h8) {
-          // A_{l-1} of 8 points x 4 jet rows from the swizzled tile: row rr of box r,
-          // 16-byte chunk (pc + 8 h8) / 8 XOR (rr mod 8)
+          // A_{l-1} of 8 points x 4 jet rows from the swizzled tile (staged: Zbar_{l-1} back in
+          // its place): row rr of box r, 16-byte chunk (pc + 8 h8) / 8 XOR (rr mod 8)
           uint32_t aw[4][4];
-          const int chunk = ((pc + 8 * h8) >> 3) ^ (rr & 7);
+          const uint32_t addr = smem_u32(at + rr * 128 + ((((pc + 8 * h8) >> 3) ^ (rr & 7)) << 4));
 #pragma unroll
-          for (int r = 0; r < 4; ++r) {
-            const uint32_t addr = smem_u32(at + r * FZ_ABOX + rr * 128 + chunk * 16);
+          for (int r = 0; r < 4; ++r)
             asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];"
                          : "=r"(aw[r][0]), "=r"(aw[r][1]), "=r"(aw[r][2]), "=r"(aw[r][3])
-                         : "r"(addr));
-          }
+                         : "r"(addr + r * FZ_ABOX));
           with_jet_mode(p.e.jet_mode, [&](auto mode) { adj_pairs8<decltype(mode)::value>(v[u], 8 * h8, aw); });
+          if constexpr (!DW) {
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+              uint32_t q[4];
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                const __nv_bfloat162 x = __floats2bfloat162_rn(v[u][r][8 * h8 + 2 * i], v[u][r][8 * h8 + 2 * i + 1]);
+                q[i] = *reinterpret_cast<const uint32_t*>(&x);
+              }
+              asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(addr + r * FZ_ABOX), "r"(q[0]), "r"(q[1]),
+                           "r"(q[2]), "r"(q[3])
+                           : "memory");
+            }
+          }
         }
-        if (mvalid) {
-          const int64_t cbase = toff(m, (int64_t)nb * BN, p.M) + pc;
-          T* zbo = reinterpret_cast<T*>(p.e.out) + cbase;
+        if (u == UNITS - 1) {   // this warp is through with the tile: its accesses before the next bulk copy's
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&z_done[ab]);
+        }
+        if (DW && mvalid) {
+          __nv_bfloat16* zbo = reinterpret_cast<__nv_bfloat16*>(p.e.out) + toff(m, (int64_t)nb * BN, p.M) + pc;
 #pragma unroll
           for (int r = 0; r < 4; ++r) st_row(zbo + 64 * r, v[u][r]);
         }
@@ -1270,10 +1395,6 @@ __device__ __forceinline__ void tc_adjdw_body(const CUtensorMap* mapW, const CUt
           if (p.e.dterms) coord_terms<UPTS>(v[u], xc, u * UPTS, p.e.dterms, p.e.jet_mode, db);
         }
       }
-      // done with this A tile: its ordinary shared loads ordered before the next bulk copy
-      // into the buffer (the mbarrier orders the generic proxy only)
-      fence_proxy_async_smem();
-      mbar_arrive(&a_empty[ab]);
       if (mvalid && p.e.dbpart) {
         float* dst = p.e.dbpart + ((int64_t)m * (p.n_tiles * PARTS) + nb * PARTS + part) * (1 + p.e.dterms);
         dst[0] = db[0];
@@ -1283,7 +1404,7 @@ __device__ __forceinline__ void tc_adjdw_body(const CUtensorMap* mapW, const CUt
       }
     }
     // this CTA's dW^T slab (its m-tile rows x all fout) as split partial (CTA index) / m_tiles
-    if (local > 0 && !*abort_flag && mbar_wait(dw_full, 0, abort_flag, p.status, p.wait_ns)) {
+    if (DW && local > 0 && !*abort_flag && mbar_wait(dw_full, 0, abort_flag, p.status, p.wait_ns)) {
       tc_fence_after();
       const int m = mb_cta * BM + rr;
       const int split = grid.bx() / p.m_tiles;
@@ -1329,16 +1450,19 @@ __device__ __forceinline__ void tc_adjdw_body(const CUtensorMap* mapW, const CUt
   }
 }
 
+template <bool DW>
 __global__ void __launch_bounds__(FZ_NT, 1)
     k_tc_adjdw(const __grid_constant__ CUtensorMap mapW, const __grid_constant__ CUtensorMap mapZ,
-               const __grid_constant__ CUtensorMap mapA, const __grid_constant__ TcParams p) {
-  tc_adjdw_body(&mapW, &mapZ, &mapA, p, SingleGrid{});
+               const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapO,
+               const __grid_constant__ TcParams p) {
+  tc_adjdw_body<DW>(&mapW, &mapZ, &mapA, &mapO, p, SingleGrid{});
 }
 
+template <bool DW>
 __global__ void __launch_bounds__(FZ_NT, 1) k_tc_adjdw_group(const TcGroupEntry* __restrict__ tab, const int n) {
   const TcGroupEntry& g = tab[group_of_block(tab, n, (int)blockIdx.x)];
-  acquire_maps(g, 3);
-  tc_adjdw_body(&g.map[0], &g.map[1], &g.map[2], g.p, GroupShare{(int)blockIdx.x - g.block0, g.grid});
+  acquire_maps(g, 4);
+  tc_adjdw_body<DW>(&g.map[0], &g.map[1], &g.map[2], &g.map[3], g.p, GroupShare{(int)blockIdx.x - g.block0, g.grid});
 }
 
 int adjdw_grid(const pinn_handle* h, int fin, int64_t NC) {
@@ -1346,6 +1470,51 @@ int adjdw_grid(const pinn_handle* h, int fin, int64_t NC) {
   const int tiles = mt * (int)(NC / TILE_COLS);
   const int per = std::max(1, std::max(h->sm_count, 1) / mt) * mt;   // a multiple of the m-tile count
   return std::max(mt, std::min(tiles, per));
+}
+
+}  // namespace
+
+namespace {
+
+template <bool DW>
+pinn_status launch_adjdw_group(pinn_handle* h, const TcGroupEntry* d_tab, int n, int blocks, cudaStream_t st) {
+  static bool attr_set = false;   // per instantiation
+  pinn_status s = reserve_smem(h, k_tc_adjdw_group<DW>, FzCfg<DW>::SMEM, attr_set, "grouped fused adjoint kernel");
+  if (s) return s;
+  k_tc_adjdw_group<DW><<<blocks, FZ_NT, FzCfg<DW>::SMEM, st>>>(d_tab, n);
+  return launch_check(h, "grouped fused adjoint");
+}
+
+template <bool DW>
+pinn_status launch_adjdw(pinn_handle* h, const CUtensorMap& w, const CUtensorMap& z, const CUtensorMap& a,
+                         const CUtensorMap& o, const TcParams& p, int grid, cudaStream_t st) {
+  if (h->tc_batch) {
+    const CUtensorMap maps[4] = {w, z, a, o};
+    return batch_add(h->tc_batch, &launch_adjdw_group<DW>, maps, 4, p, grid);
+  }
+  static bool attr_set = false;   // per instantiation
+  pinn_status s = reserve_smem(h, k_tc_adjdw<DW>, FzCfg<DW>::SMEM, attr_set, "fused adjoint kernel");
+  if (s) return s;
+  k_tc_adjdw<DW><<<grid, FZ_NT, FzCfg<DW>::SMEM, st>>>(w, z, a, o, p);
+  return launch_check(h, "fused adjoint");
+}
+
+}  // namespace
+
+namespace {
+
+// The BF16 tanh adjoint of a layer whose weight gradient runs on its own (fan-out above 256).
+pinn_status adj_staged(pinn_handle* h, const void* WT, const void* Zbar, int fin, int fout, int64_t NC,
+                       const EpiArgs& e, cudaStream_t st) {
+  CUtensorMap mw, mz, ma, mo;
+  const uint64_t nt = (uint64_t)(NC / TILE_COLS);
+  if (!make_map(&mw, WT, false, fout, fin, 64, BM)) return map_err(h, "adjoint weights");
+  if (!make_map3(&mz, Zbar, false, TILE_COLS, fout, nt, 64, 64)) return map_err(h, "adjoint input");
+  if (!make_map3(&ma, e.ain, false, TILE_COLS, fin, nt, 64, BM)) return map_err(h, "adjoint activations");
+  if (!make_map3(&mo, e.out, false, TILE_COLS, fin, nt, 64, BM)) return map_err(h, "adjoint output");
+  TcParams p = base_params(fin, (int)NC, fout, NC, 64, h->d_status);
+  p.e = e;
+  return launch_adjdw<false>(h, mw, mz, ma, mo, p, grid_for(h, p.m_tiles * p.n_tiles), st);
 }
 
 }  // namespace
@@ -1363,11 +1532,12 @@ int tc_adjdw_splits(const pinn_handle* h, int fin, int64_t NC) {
 
 pinn_status tc_gemm_adjdw(pinn_handle* h, const void* WT, const void* Zbar, const void* Ain, int fin, int fout,
                           int64_t NC, const EpiArgs& e, float* dwpart, int nsplit, cudaStream_t st) {
-  CUtensorMap mw, mz, ma;
+  CUtensorMap mw, mz, ma, mo;
   const uint64_t nt = (uint64_t)(NC / TILE_COLS);
   if (!make_map(&mw, WT, false, fout, fin, 64, BM)) return map_err(h, "fused adjoint weights");
   if (!make_map3(&mz, Zbar, false, TILE_COLS, fout, nt, 64, 64)) return map_err(h, "fused adjoint input");
   if (!make_map3(&ma, Ain, false, TILE_COLS, fin, nt, 64, BM)) return map_err(h, "fused adjoint activations");
+  if (!make_map3(&mo, e.out, false, TILE_COLS, fin, nt, 64, BM)) return map_err(h, "fused adjoint output");
   TcParams p = base_params(fin, (int)NC, fout, NC, 64, h->d_status);
   p.e = e;
   p.out32 = dwpart;
@@ -1377,28 +1547,8 @@ pinn_status tc_gemm_adjdw(pinn_handle* h, const void* WT, const void* Zbar, cons
     return PINN_ERR_INVALID_ARG;
   }
   p.nsplit = nsplit;
-  if (h->tc_batch) {
-    const CUtensorMap maps[3] = {mw, mz, ma};
-    return batch_add(h->tc_batch, &launch_adjdw_group, maps, 3, p, grid);
-  }
-  static bool attr_set = false;
-  pinn_status s = reserve_smem(h, k_tc_adjdw, FZ_SMEM, attr_set, "fused adjoint kernel");
-  if (s) return s;
-  k_tc_adjdw<<<grid, FZ_NT, FZ_SMEM, st>>>(mw, mz, ma, p);
-  return launch_check(h, "fused adjoint");
+  return launch_adjdw<true>(h, mw, mz, ma, mo, p, grid, st);
 }
-
-namespace {
-
-pinn_status launch_adjdw_group(pinn_handle* h, const TcGroupEntry* d_tab, int n, int blocks, cudaStream_t st) {
-  static bool attr_set = false;
-  pinn_status s = reserve_smem(h, k_tc_adjdw_group, FZ_SMEM, attr_set, "grouped fused adjoint kernel");
-  if (s) return s;
-  k_tc_adjdw_group<<<blocks, FZ_NT, FZ_SMEM, st>>>(d_tab, n);
-  return launch_check(h, "grouped fused adjoint");
-}
-
-}  // namespace
 
 // ==== the whole hidden forward in one kernel (BF16 tanh, every width <= 256) ===========
 //
@@ -1727,16 +1877,9 @@ __global__ void __launch_bounds__(FF_NT, 1) k_tc_fwd_all(const __grid_constant__
             mbar_arrive(&accr[h]);
           }
           if (last) {
-            if (rows(l, h) && m < M) {
-              const int pc = part * (UNITS * UPTS);
-              __nv_bfloat16* ao = p.a_last + toff(m, (int64_t)nb * BN, M) + pc;
-              __nv_bfloat16* al = p.alo_last + loff(m, (int64_t)nb * TILE_PTS, M) + pc;
-#pragma unroll
-              for (int u = 0; u < UNITS; ++u) {
-#pragma unroll
-                for (int r = 0; r < 4; ++r) st_global_256(ao + UPTS * u + 64 * r, hi[u][r]);
-                st_global_256(al + UPTS * u, lo[u]);
-              }
+            if (rows(l, h)) {
+              store_pairs(p.a_last, hi, m, nb, M, part * (UNITS * UPTS));
+              store_lo_pairs(p.alo_last, lo, m, nb, M, part * (UNITS * UPTS));
             }
             continue;
           }

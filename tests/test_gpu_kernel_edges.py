@@ -105,3 +105,22 @@ def test_fused_forward_edges(cuda_lib, widths, ff, n_res):
     if Bd is not None:
         net.set_ff_matrix(B)
     assert torch.equal(net.loss(params, db, prob), res[0][0])
+
+
+@pytest.mark.parametrize("pde,widths,ff", [
+    (PDE_BURGERS, [264, 272], 0),             # m-tiles of 8 rows, raw first layer (coordinate terms)
+    (PDE_NS, [512, 304, 264], 16),            # even and odd m-tile counts
+    (PDE_MAXWELL, [40, 1024, 16], 0),         # one m-tile below a wide layer, K of 16 chunks
+])
+@pytest.mark.parametrize("n_res", [1, 7000])  # one tile, and more units than two rounds of every SM
+def test_wide_layer_edges(cuda_lib, pde, widths, ff, n_res):
+    """The per-layer forward and the staged adjoint of layers above 256 wide against the oracle:
+    total loss and whole gradient (the residual of a single point may cancel below the
+    precision's tolerance)."""
+    spec = NetSpec(pde, 3 if pde == PDE_MAXWELL else 2, 1 if pde == PDE_BURGERS else 3, widths, ff_m=ff, ff_sigma=1.0)
+    p, B, prob = init_params(spec, 95, 0.2), ff_matrix(spec, 96), Problem(0.02, 0.3, 2.0, 5.0)
+    b = make_batch(pde, n_res, 30, 20, 97, 98)
+    gt, gg = run_gpu(spec, p, B, b, prob, "bf16")
+    rt, rg = run_oracle(spec, p, B, b, prob, chunk=4096)
+    assert abs(gt[0] - rt[0]) <= TOL["bf16"] * abs(rt[0])
+    assert np.linalg.norm(gg - rg) <= TOL["bf16"] * np.linalg.norm(rg)
