@@ -141,7 +141,7 @@ void launch_first_layer(const float* x_res, const float* x_ic, const float* x_bc
 
 struct EpiArgs {
   const float* bias;      // fwd: bias of this layer [M]
-  void* out;              // fwd: A_l^T, adj: Zbar_{l-1}^T (compute type)
+  void* out;              // fwd: A_l^T, adj: Zbar_{l-1}^T (compute type; tensor cores: nullptr = not stored)
   void* alo_out;          // fwd, BF16: low half of A_l's value rows [M][NP] (else nullptr)
   const void* alo_in;     // fwd, CUDA-core BF16 path: low half of the input's value rows [K][NP]
   const void* ain;        // adj: A_{l-1}^T (compute type), the output jet of the layer below

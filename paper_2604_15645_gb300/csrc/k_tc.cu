@@ -557,8 +557,9 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA, const CUte
       int mb, nb, k0, k1;
       coords(t, mb, nb, k0, k1);
       const int buf = DW2 ? 0 : local & 1;
-      if (!mbar_wait(&acc_full[buf], DW2 ? ((uint32_t)local & 1) : ((uint32_t)(local >> 1) & 1), abort_flag,
-                     p.status, p.wait_ns)) break;
+      const bool got = mbar_wait(&acc_full[buf], DW2 ? ((uint32_t)local & 1) : ((uint32_t)(local >> 1) & 1), abort_flag,
+                                 p.status, p.wait_ns);
+      if (__any_sync(0xffffffffu, !got)) break;   // (the warp's loads and shuffles are collective)
       tc_fence_after();
       for (int half = 0; half < (DW2 ? 2 : 1); ++half) {
       const int m = mb * MROWS + half * BM + row;
@@ -643,9 +644,11 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA, const CUte
               for (int r = 0; r < 4; ++r) v[r][i] = zb[r];
             }
           }
-          T* zbo = reinterpret_cast<T*>(p.e.out) + cbase;
+          if (p.e.out) {
+            T* zbo = reinterpret_cast<T*>(p.e.out) + cbase;
 #pragma unroll
-          for (int r = 0; r < 4; ++r) st_row(zbo + 64 * r, v[r]);
+            for (int r = 0; r < 4; ++r) st_row(zbo + 64 * r, v[r]);
+          }
           if constexpr (TF32) {
             if (p.e.out_pm) store_pm8(reinterpret_cast<float*>(p.e.out_pm), (int64_t)nb * BN + pc, p.M, m, v);
           }
@@ -1223,7 +1226,7 @@ __device__ __forceinline__ void tc_adjdw_body(const CUtensorMap* mapW, const CUt
         const int ab = out % FZ_ABUF;
         ok = mbar_wait(&z_done[ab], (uint32_t)(out / FZ_ABUF) & 1, abort_flag, p.status, p.wait_ns);
         if (!ok) return;
-        if constexpr (!DW) {
+        if (!DW && p.e.out) {
           int mb, nb;
           coords(t_out, mb, nb);
           const uint8_t* at = abase + ab * FZ_AT;
@@ -1364,7 +1367,7 @@ __device__ __forceinline__ void tc_adjdw_body(const CUtensorMap* mapW, const CUt
                          : "=r"(aw[r][0]), "=r"(aw[r][1]), "=r"(aw[r][2]), "=r"(aw[r][3])
                          : "r"(addr + r * FZ_ABOX));
           with_jet_mode(p.e.jet_mode, [&](auto mode) { adj_pairs8<decltype(mode)::value>(v[u], 8 * h8, aw); });
-          if constexpr (!DW) {
+          if (!DW && p.e.out) {
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
               uint32_t q[4];
@@ -1384,7 +1387,7 @@ __device__ __forceinline__ void tc_adjdw_body(const CUtensorMap* mapW, const CUt
           __syncwarp();
           if (lane == 0) mbar_arrive(&z_done[ab]);
         }
-        if (DW && mvalid) {
+        if (DW && mvalid && p.e.out) {
           __nv_bfloat16* zbo = reinterpret_cast<__nv_bfloat16*>(p.e.out) + toff(m, (int64_t)nb * BN, p.M) + pc;
 #pragma unroll
           for (int r = 0; r < 4; ++r) st_row(zbo + 64 * r, v[u][r]);
@@ -1511,7 +1514,8 @@ pinn_status adj_staged(pinn_handle* h, const void* WT, const void* Zbar, int fin
   if (!make_map(&mw, WT, false, fout, fin, 64, BM)) return map_err(h, "adjoint weights");
   if (!make_map3(&mz, Zbar, false, TILE_COLS, fout, nt, 64, 64)) return map_err(h, "adjoint input");
   if (!make_map3(&ma, e.ain, false, TILE_COLS, fin, nt, 64, BM)) return map_err(h, "adjoint activations");
-  if (!make_map3(&mo, e.out, false, TILE_COLS, fin, nt, 64, BM)) return map_err(h, "adjoint output");
+  mo = ma;
+  if (e.out && !make_map3(&mo, e.out, false, TILE_COLS, fin, nt, 64, BM)) return map_err(h, "adjoint output");
   TcParams p = base_params(fin, (int)NC, fout, NC, 64, h->d_status);
   p.e = e;
   return launch_adjdw<false>(h, mw, mz, ma, mo, p, grid_for(h, p.m_tiles * p.n_tiles), st);
@@ -1537,7 +1541,7 @@ pinn_status tc_gemm_adjdw(pinn_handle* h, const void* WT, const void* Zbar, cons
   if (!make_map(&mw, WT, false, fout, fin, 64, BM)) return map_err(h, "fused adjoint weights");
   if (!make_map3(&mz, Zbar, false, TILE_COLS, fout, nt, 64, 64)) return map_err(h, "fused adjoint input");
   if (!make_map3(&ma, Ain, false, TILE_COLS, fin, nt, 64, BM)) return map_err(h, "fused adjoint activations");
-  if (!make_map3(&mo, e.out, false, TILE_COLS, fin, nt, 64, BM)) return map_err(h, "fused adjoint output");
+  mo = ma;   // (not used: this form stores from registers)
   TcParams p = base_params(fin, (int)NC, fout, NC, 64, h->d_status);
   p.e = e;
   p.out32 = dwpart;
