@@ -53,20 +53,21 @@ constexpr uint64_t WAIT_NS = 2000000000ull;   // default bound on any single wai
 
 enum TcMode { TC_FWD = 0, TC_ADJ = 1, TC_DW = 2, TC_STORE = 3 };
 
-// Shared-memory matrix descriptor (tcgen05), 128-byte swizzle, version 1.
+// Shared-memory matrix descriptor (tcgen05), 128- or 64-byte swizzle, version 1.
+template <int SWIZZLE = 128>
 __device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
   uint64_t d = 0;
   d |= (uint64_t)((saddr >> 4) & 0x3FFF);
   d |= (uint64_t)((lbo >> 4) & 0x3FFF) << 16;
   d |= (uint64_t)((sbo >> 4) & 0x3FFF) << 32;
   d |= (uint64_t)1 << 46;   // descriptor version for tcgen05
-  d |= (uint64_t)2 << 61;   // SWIZZLE_128B
+  d |= (uint64_t)(SWIZZLE == 128 ? 2 : 4) << 61;   // SWIZZLE_128B / SWIZZLE_64B
   return d;
 }
 // Instruction descriptor: FP32 accumulate, A/B format (1 = BF16, 2 = TF32),
-// A K-major, B K-major (b_mn = 0) or MN-major (b_mn = 1), N columns, M = BM.
-__host__ __device__ constexpr uint32_t make_idesc(uint32_t fmt, uint32_t b_mn, uint32_t n = BN) {
-  return (1u << 4) | (fmt << 7) | (fmt << 10) | (b_mn << 16) | ((n >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+// A K-major, B K-major (b_mn = 0) or MN-major (b_mn = 1), N columns, M rows.
+__host__ __device__ constexpr uint32_t make_idesc(uint32_t fmt, uint32_t b_mn, uint32_t n = BN, uint32_t m = BM) {
+  return (1u << 4) | (fmt << 7) | (fmt << 10) | (b_mn << 16) | ((n >> 3) << 17) | ((m >> 4) << 24);
 }
 
 struct TcParams {
@@ -115,39 +116,65 @@ __device__ __forceinline__ int group_of_block(const TcGroupEntry* __restrict__ t
 // Where a CTA sits in the launch: the hardware indices of a single launch (read where
 // used, as a plain kernel would), or its share of a grouped launch.
 struct SingleGrid {
+  static constexpr bool PAIR = false;
   __device__ __forceinline__ int bx() const { return (int)blockIdx.x; }
   __device__ __forceinline__ int gdim() const { return (int)gridDim.x; }
 };
 struct GroupShare {
+  static constexpr bool PAIR = false;
   int b, g;
   __device__ __forceinline__ int bx() const { return b; }
   __device__ __forceinline__ int gdim() const { return g; }
 };
 
-template <bool TF32, int MODE, bool SPLIT>
+// A single launch in clusters of two CTAs: neighbours, which hold two m-tiles of the same
+// column tile and run their MMAs as one of 256 rows (cta_group::2), each staging half of
+// the column operand.
+struct PairGrid : SingleGrid {
+  static constexpr bool PAIR = true;
+};
+// Last step of a CTA of a pair: the other one arrives at this one's barriers and its MMAs
+// read this one's shared memory, so neither leaves before both are done.  (After an abort
+// MMAs, copies and arrivals that are still on their way take microseconds: wait them out.)
+__device__ __forceinline__ void pair_leave(volatile int* abort_flag) {
+  cluster_sync();
+  if (threadIdx.x == 0 && *abort_flag) {
+    const uint64_t t0 = gtimer();
+    while (gtimer() - t0 < 1000000ull) {}
+  }
+  cluster_sync();
+}
+
+template <bool TF32, int MODE, bool SPLIT, bool PAIR = false>
 struct Cfg {
   static constexpr int ES = TF32 ? 4 : 2;
   static constexpr int BKE = 128 / ES;            // K elements per stage (one 128-byte swizzle row)
   static constexpr int UK = TF32 ? 8 : 16;        // K per MMA instruction
   static constexpr int A_BYTES = BM * 128;        // 16 KB
-  static constexpr int B_BYTES = BN * 128;        // 32 KB
+  static constexpr int B_BYTES = BN * 128 / (PAIR ? 2 : 1);   // 32 KB (pair: half of the columns)
   // TF32 forward / adjoint: B from the point-major copy (K-major, 2-D map), its low
   // half computed in shared memory (one B-sized buffer).
   static constexpr bool KPM = TF32 && (MODE == TC_FWD || MODE == TC_ADJ);
   static constexpr int BLOC_BYTES = KPM ? B_BYTES : 0;
   static constexpr int CVT_WARPS = KPM ? 2 : 0;
-  static constexpr int NTHREADS = 64 + 32 * (EPI_WARPS + CVT_WARPS);
+  static constexpr int NTHREADS = 64 + 32 * (EPI_WARPS + (PAIR ? 1 : CVT_WARPS));
+  // Pair: outputs leave by bulk tensor stores through these 128 x 64-point buffers.
+  static constexpr int OUT_BUFS = PAIR ? 3 : 0, OUT_BYTES = BM * 128;
   // BF16 forward: low half of the input's value rows, 64 MN-major columns per stage.
   static constexpr bool VLO = (MODE == TC_FWD) && !TF32;
+  // (Pair: 32 of them, and the same 32 value columns of the input for a low half of the
+  // weights that is limited to the value rows: a CTA provides half of every MMA's columns.)
   static constexpr int BLO_BYTES = VLO ? TILE_PTS * 128 : 0;   // 8 KB
+  static constexpr int V_BYTES = BLO_BYTES / 2;
   static constexpr int STAGE = A_BYTES * (SPLIT ? 2 : 1) + B_BYTES + BLO_BYTES;
   static constexpr int STAGES = (MODE == TC_FWD || SPLIT) ? 3 : 4;
-  static_assert(STAGES * STAGE + BLOC_BYTES + 1024 + 256 <= 227 * 1024, "shared memory budget");
+  static_assert(STAGES * STAGE + BLOC_BYTES + OUT_BUFS * OUT_BYTES + 1024 + 256 <= 227 * 1024, "shared memory budget");
   static constexpr bool B_MN = (MODE != TC_DW) && !KPM;
   static constexpr int BOXN = 128 / ES;           // MN-major box width (columns)
-  static constexpr int NBOX = BN / BOXN;
+  static constexpr int NBOX = BN / BOXN / (PAIR ? 2 : 1);
   static constexpr int BOX_BYTES = BKE * 128;     // one MN-major box: BKE rows of 128 bytes
-  static constexpr size_t SMEM = (size_t)STAGES * STAGE + BLOC_BYTES + 1024 /*align*/ + 256 /*barriers*/;
+  static constexpr size_t SMEM =
+      (size_t)STAGES * STAGE + BLOC_BYTES + OUT_BUFS * OUT_BYTES + 1024 /*align*/ + 256 /*barriers*/;
 };
 
 // Point-major copy [NC][M] of one thread's 8 points x 4 rows of feature m: column
@@ -285,8 +312,12 @@ __device__ __forceinline__ void coord_terms(const float (&v)[4][N], const float 
 template <bool TF32, int MODE, bool SPLIT, bool SINE, typename Grid>
 __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA, const CUtensorMap* mapA2,
                                              const CUtensorMap* mapB, const CUtensorMap* mapBlo, const TcParams& p,
-                                             const Grid grid) {
-  using C = Cfg<TF32, MODE, SPLIT>;
+                                             const Grid grid, const CUtensorMap* mapV = nullptr,
+                                             const CUtensorMap* mapO = nullptr, const CUtensorMap* mapOlo = nullptr) {
+  constexpr bool PAIR = Grid::PAIR;
+  static_assert(!PAIR || (MODE == TC_FWD && !TF32 && !SINE), "pairs run the BF16 tanh forward");
+  using C = Cfg<TF32, MODE, SPLIT, PAIR>;
+  const int rank = PAIR ? (int)(blockIdx.x & 1) : 0;
   using T = typename std::conditional<TF32, float, __nv_bfloat16>::type;
   // weight gradient with 256-row tiles: two 128-row accumulators (TMEM columns 0..255 and
   // 256..511) share each staged B operand, so the B rows are read once for 256 output
@@ -298,14 +329,17 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA, const CUte
   // hide the address space and turn every shared access below into a generic one)
   uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   uint8_t* blo = smem + C::STAGES * C::STAGE;          // TF32 B_lo buffer (BLOC_BYTES)
-  uint64_t* full = reinterpret_cast<uint64_t*>(blo + C::BLOC_BYTES);
+  uint8_t* outb = blo + C::BLOC_BYTES;                 // pair: output buffers
+  uint64_t* full = reinterpret_cast<uint64_t*>(outb + C::OUT_BUFS * C::OUT_BYTES);
   uint64_t* empty = full + C::STAGES;
   uint64_t* acc_full = empty + C::STAGES;
   uint64_t* acc_empty = acc_full + 2;
   uint64_t* lo_full = acc_empty + 2;                  // converter -> MMA: B_lo ready
   uint64_t* lo_empty = lo_full + 1;                   // MMA -> converter: B_lo consumed
   uint64_t* never = lo_empty + 1;                     // test hook (p.stall): no thread arrives on it
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(never + 1);
+  uint64_t* out_full = never + 1;                     // [OUT_BUFS] epilogue -> stores: buffer written
+  uint64_t* out_read = out_full + C::OUT_BUFS;        // [OUT_BUFS] stores -> epilogue: buffer read
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(out_read + C::OUT_BUFS);
   volatile int* inflight = abort_flag + 1;             // [STAGES]: parity+1 of an armed, unconsumed stage
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(const_cast<int*>(inflight + C::STAGES));
 
@@ -318,21 +352,24 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA, const CUte
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&acc_full[b], 1);
-      mbar_init(&acc_empty[b], 32 * EPI_WARPS);
+      mbar_init(&acc_empty[b], PAIR ? 2 * EPI_WARPS : 32 * EPI_WARPS);   // (pair: both CTAs' warps, at the first one's)
     }
     mbar_init(lo_full, 1);
     mbar_init(lo_empty, 1);
     mbar_init(never, 1);
+    for (int b = 0; b < C::OUT_BUFS; ++b) {
+      mbar_init(&out_full[b], EPI_WARPS);
+      mbar_init(&out_read[b], 1);
+    }
     *abort_flag = 0;
     fence_mbar_init();
   }
   if (warp == 1) {   // allocate 2 x 256 TMEM columns (whole warp)
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                 "r"(2 * BN));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    tmem_alloc<PAIR>(tmem_slot, 2 * BN);
   }
   tc_fence_before();
   __syncthreads();
+  if (PAIR) cluster_sync();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
@@ -365,9 +402,26 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA, const CUte
           uint8_t* sa = smem + stage * C::STAGE;
           uint8_t* sa2 = sa + C::A_BYTES;
           uint8_t* sb = sa + C::A_BYTES * (SPLIT ? 2 : 1);
+          const int kx = kb * C::BKE;
+          if constexpr (PAIR) {
+            // both CTAs' copies complete at the first one's barrier: it issues the MMAs
+            const uint32_t bar = cta_addr(&full[stage], 0);
+            if (rank == 0) {
+              mbar_expect_tx(&full[stage], 2 * (C::STAGE - (p.wlo_values_only ? 0 : C::V_BYTES)));
+              inflight[stage] = (int)phase + 1;
+            }
+            tma_load_2d_pair(sa, mapA, bar, kx, mb * BM);
+            tma_load_2d_pair(sa2, mapA2, bar, kx, mb * BM);
+#pragma unroll
+            for (int j = 0; j < C::NBOX; ++j)
+              tma_load_3d_pair(sb + j * C::BOX_BYTES, mapB, bar, (C::NBOX * rank + j) * C::BOXN, kx, nb);
+            tma_load_3d_pair(sb + C::B_BYTES, mapBlo, bar, rank * (TILE_PTS / 2), kx, nb);
+            if (p.wlo_values_only) tma_load_3d_pair(sb + C::B_BYTES + C::V_BYTES, mapV, bar, rank * (TILE_PTS / 2), kx, nb);
+            if (++stage == C::STAGES) { stage = 0; phase ^= 1; }
+            continue;
+          }
           mbar_expect_tx(&full[stage], C::STAGE);
           inflight[stage] = (int)phase + 1;
-          const int kx = kb * C::BKE;
           if (C::KPM) {
             // A: weights [M][K]; B: point-major jets [NC][K], columns nb*BN.. (both 2-D, K-major)
             tma_load_2d(sa, mapA, &full[stage], kx, mb * BM);
@@ -396,11 +450,17 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA, const CUte
           if (++stage == C::STAGES) { stage = 0; phase ^= 1; }
         }
       }
+      if (PAIR)   // the last arrivals land before this CTA may leave
+        for (int s = 0; s < C::STAGES; ++s) {
+          if (!mbar_wait(&empty[stage], phase ^ 1, abort_flag, p.status, p.wait_ns)) break;
+          if (++stage == C::STAGES) { stage = 0; phase ^= 1; }
+        }
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issuer
-    if (lane == 0) {
-      constexpr uint32_t idesc = make_idesc(TF32 ? 2u : 1u, C::B_MN ? 1u : 0u);
+    if (lane == 0 && rank == 0) {
+      constexpr uint32_t MR = PAIR ? 2 * BM : BM;
+      constexpr uint32_t idesc = make_idesc(TF32 ? 2u : 1u, C::B_MN ? 1u : 0u, BN, MR);
       int stage = 0;
       uint32_t phase = 0, lo_phase = 0;
       int local = 0;
@@ -412,7 +472,7 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA, const CUte
         coords(t, mb, nb, k0, k1);
         const int buf = DW2 ? 0 : local & 1;
         const uint32_t par = DW2 ? ((uint32_t)local & 1) : ((uint32_t)(local >> 1) & 1);
-        if (!mbar_wait(&acc_empty[buf], par ^ 1, abort_flag, p.status, p.wait_ns)) break;
+        if (!mbar_wait<PAIR>(&acc_empty[buf], par ^ 1, abort_flag, p.status, p.wait_ns)) break;
         tc_fence_after();
         const uint32_t d = tmem_base + buf * BN;
         bool ok = true;
@@ -428,7 +488,17 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA, const CUte
             const uint64_t ad = make_desc(sa + kk * 32, 16, 1024);
             const uint64_t bd = C::B_MN ? make_desc(sb + kk * C::UK * 128, C::BOX_BYTES, 1024)
                                         : make_desc(sb + kk * 32, 16, 1024);
-            tc_mma<TF32>(d, ad, bd, idesc, (kb > k0 || kk > 0) ? 1u : 0u);
+            tc_mma<TF32, PAIR>(d, ad, bd, idesc, (kb > k0 || kk > 0) ? 1u : 0u);
+            if constexpr (PAIR) {
+              // the same sums as below; the 64 value columns are 32 of each CTA (64-byte swizzle)
+              constexpr uint32_t idesc64 = make_idesc(1u, 1u, TILE_PTS, MR);
+              const uint32_t sl = sb + C::B_BYTES + kk * C::UK * 64;
+              const uint64_t ad2 = make_desc(sa2 + kk * 32, 16, 1024);
+              if (p.wlo_values_only) tc_mma<TF32, PAIR>(d, ad2, make_desc<64>(sl + C::V_BYTES, 512, 512), idesc64, 1u);
+              else tc_mma<TF32, PAIR>(d, ad2, bd, idesc, 1u);
+              tc_mma<TF32, PAIR>(d, ad, make_desc<64>(sl, 512, 512), idesc64, 1u);
+              continue;
+            }
             if constexpr (DW2) {
               // the second 128 output rows, same B operand, into TMEM columns 256..511
               tc_mma<TF32>(d + BN, make_desc(sa2 + kk * 32, 16, 1024), bd, idesc, (kb > k0 || kk > 0) ? 1u : 0u);
@@ -454,11 +524,11 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA, const CUte
             tc_commit(lo_empty);
             lo_phase ^= 1;
           }
-          tc_commit(&empty[stage]);
+          tc_commit<PAIR>(&empty[stage]);
           if (++stage == C::STAGES) { stage = 0; phase ^= 1; }
         }
         if (!ok) break;
-        tc_commit(&acc_full[buf]);
+        tc_commit<PAIR>(&acc_full[buf]);
       }
     }
   } else if (C::KPM && warp >= 2 + EPI_WARPS) {
@@ -510,6 +580,28 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA, const CUte
       }
       if (!ok) break;
     }
+  } else if (PAIR && warp >= 2 + EPI_WARPS) {
+    // ---------------------------------------------------------------- output stores (pair)
+    if (lane == 0) {
+      const int items = p.e.alo_out ? 5 : 4;              // jet rows, then the value rows' low half
+      int b = 0;
+      uint32_t ph = 0;
+      bool ok = true;
+      for (int t = grid.bx(); t < total && ok; t += grid.gdim()) {
+        int mb, nb, k0, k1;
+        coords(t, mb, nb, k0, k1);
+        for (int i = 0; i < items; ++i) {
+          ok = mbar_wait(&out_full[b], ph, abort_flag, p.status, p.wait_ns);
+          if (!ok) break;
+          tma_store_3d(i < 4 ? mapO : mapOlo, outb + b * C::OUT_BYTES, i < 4 ? TILE_PTS * i : 0, mb * BM, nb);
+          bulk_commit();
+          bulk_wait_read0();
+          mbar_arrive(&out_read[b]);
+          if (++b == C::OUT_BUFS) { b = 0; ph ^= 1; }
+        }
+      }
+      bulk_wait0();
+    }
   } else if (warp < 2 + EPI_WARPS) {
     // ---------------------------------------------------------------- epilogue
     // Warp part `part` of a lane quadrant handles points 32 part .. 32 part + 31 of the
@@ -552,8 +644,11 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA, const CUte
     if constexpr (MODE == TC_ADJ && !SINE) {
       if (grid.bx() < total) load_z(grid.bx(), 0);
     }
+    [[maybe_unused]] int ob = 0;                          // pair: the next output buffer, its uses' parity
+    [[maybe_unused]] uint32_t oph = 0;
+    bool left = false;                                   // an output buffer's wait expired
     int local = 0;
-    for (int t = grid.bx(); t < total; t += grid.gdim(), ++local) {
+    for (int t = grid.bx(); t < total && !left; t += grid.gdim(), ++local) {
       int mb, nb, k0, k1;
       coords(t, mb, nb, k0, k1);
       const int buf = DW2 ? 0 : local & 1;
@@ -701,13 +796,42 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA, const CUte
           tmem_wait_ld();
           if (u == UNITS - 1) {
             tc_fence_before();
-            mbar_arrive(&acc_empty[buf]);
+            if constexpr (PAIR) {
+              __syncwarp();
+              if (lane == 0) mbar_arrive_cta(&acc_empty[buf], 0);
+            } else {
+              mbar_arrive(&acc_empty[buf]);
+            }
           }
           with_jet_mode(p.e.jet_mode,
                         [&](auto mode) { fwd_pairs<decltype(mode)::value>(v, bias, w[u], lo[u], 0xffffffffu); });
         }
-        store_pairs(reinterpret_cast<T*>(p.e.out), w, m, nb, p.M, unit_col(0));
-        if (p.e.alo_out) store_lo_pairs(reinterpret_cast<T*>(p.e.alo_out), lo, m, nb, p.M, unit_col(0));
+        if constexpr (PAIR) {
+          // 64 bytes of each row into the swizzled buffer: 16-byte chunk (32 part + 16 u + 8 q) / 8
+          auto put = [&](const uint32_t (&a)[8], const uint32_t (&b)[8]) {
+            const bool ok = mbar_wait(&out_read[ob], oph ^ 1, abort_flag, p.status, p.wait_ns);
+            if (__any_sync(0xffffffffu, !ok)) { left = true; return; }
+            const uint32_t at = smem_u32(outb + ob * C::OUT_BYTES + row * 128);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              const uint32_t* x = (q < 2 ? a : b) + 4 * (q & 1);
+              asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(at + (((part * 4 + q) ^ (row & 7)) << 4)),
+                           "r"(x[0]), "r"(x[1]), "r"(x[2]), "r"(x[3])
+                           : "memory");
+            }
+            fence_proxy_async_smem();                   // these writes before the bulk store's reads
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&out_full[ob]);
+            if (++ob == C::OUT_BUFS) { ob = 0; oph ^= 1; }
+          };
+#pragma unroll
+          for (int r = 0; r < 4; ++r)
+            if (!left) put(w[0][r], w[1][r]);
+          if (p.e.alo_out && !left) put(lo[0], lo[1]);
+        } else {
+          store_pairs(reinterpret_cast<T*>(p.e.out), w, m, nb, p.M, unit_col(0));
+          if (p.e.alo_out) store_lo_pairs(reinterpret_cast<T*>(p.e.alo_out), lo, m, nb, p.M, unit_col(0));
+        }
       } else if constexpr (PIPE) {
         float va[4][UPTS], vb[4][UPTS];
         issue(0, va);
@@ -758,9 +882,10 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA, const CUte
   }
   tc_fence_before();
   __syncthreads();
+  if (PAIR) pair_leave(abort_flag);
   if (warp == 1) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(2 * BN));
+    tmem_free<PAIR>(tmem_base, 2 * BN);
   }
 }
 
@@ -770,6 +895,23 @@ __global__ void __launch_bounds__(Cfg<TF32, MODE, SPLIT>::NTHREADS, 1)
               const __grid_constant__ CUtensorMap mapB, const __grid_constant__ CUtensorMap mapBlo,
               const __grid_constant__ TcParams p) {
   tc_gemm_body<TF32, MODE, SPLIT, SINE>(&mapA, &mapA2, &mapB, &mapBlo, p, SingleGrid{});
+}
+
+// The BF16 tanh forward in pairs.  Launched alone, a 128 x 256 unit of a 512-wide layer is
+// bound by the path of shared memory: 24 KB of operands per K step and 72 KB of copies per
+// stage, a cycle per 128 bytes.  As a pair each CTA stages half of the columns (56 KB) and its
+// MMAs read half of them (18 KB); the smaller stages leave room for output buffers, from which
+// the tile leaves by bulk tensor stores.  Same sums in the same order.  Forward launches,
+// ms: Maxwell 5x512 at 294,912 points 3.38 -> 3.09, 8x512 cavity at 1,064,960 23.4 -> 22.2.
+// (Pairs that store from registers: 3.28 and 24.3.)  What bounds it now: neither the MMAs (no
+// faster with the low half of the weights on the value rows only) nor HBM (57%); without its
+// epilogue the unpaired kernel took 0.71 of its time.
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Cfg<false, TC_FWD, true, true>::NTHREADS, 1)
+    k_tc_fwd_pair(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapA2,
+                  const __grid_constant__ CUtensorMap mapB, const __grid_constant__ CUtensorMap mapBlo,
+                  const __grid_constant__ CUtensorMap mapV, const __grid_constant__ CUtensorMap mapO,
+                  const __grid_constant__ CUtensorMap mapOlo, const __grid_constant__ TcParams p) {
+  tc_gemm_body<false, TC_FWD, true, false>(&mapA, &mapA2, &mapB, &mapBlo, p, PairGrid{}, &mapV, &mapO, &mapOlo);
 }
 
 // Grouped launch: the GEMMs of several networks (or layers) side by side, each entry of
@@ -807,7 +949,7 @@ bool make_map(CUtensorMap* m, const void* base, bool tf32, uint64_t cols, uint64
 // jet matrices, 64 for value-row low halves), box [1][box_rows][box_cols], 128-byte
 // swizzle, zero fill out of bounds.
 bool make_map3(CUtensorMap* m, const void* base, bool tf32, uint64_t tcols, uint64_t rows, uint64_t ntiles,
-               uint32_t box_cols, uint32_t box_rows) {
+               uint32_t box_cols, uint32_t box_rows, CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_128B) {
   if (!g_encode) return false;
   const uint32_t es = tf32 ? 4 : 2;
   cuuint64_t dims[3] = {tcols, rows, ntiles};
@@ -816,7 +958,7 @@ bool make_map3(CUtensorMap* m, const void* base, bool tf32, uint64_t tcols, uint
   cuuint32_t estr[3] = {1, 1, 1};
   CUresult r = g_encode(m, tf32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3,
                         const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                        CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                        swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
 }
@@ -910,6 +1052,10 @@ pinn_status launch(pinn_handle* h, const CUtensorMap& a, const CUtensorMap& a2, 
   return launch_check(h, "tcgen05 kernel");
 }
 
+// Whether a launch runs in pairs: two m-tiles of a column tile side by side, so an even
+// number of them (and not in a grouped launch, whose entries start at any block).
+bool in_pairs(const pinn_handle* h, const TcParams& p) { return !h->tc_batch && p.m_tiles % 2 == 0 && h->sm_count >= 2; }
+
 int grid_for(const pinn_handle* h, int tiles) { return std::max(1, std::min(tiles, std::max(h->sm_count, 1))); }
 
 }  // namespace
@@ -999,8 +1145,26 @@ pinn_status fwd_impl(pinn_handle* h, const void* W, const void* Wlo, const void*
   p.e = e;
   p.wlo_values_only = (!TF32 && (h->spec.flags & PINN_FLAG_BF16_VALUE_SPLIT)) ? 1 : 0;
   const int grid = grid_for(h, p.m_tiles * p.n_tiles);
-  if constexpr (!TF32)
+  if constexpr (!TF32) {
     if (h->act == PINN_ACT_SINE) return launch<TF32, TC_FWD, true, true>(h, ma, ma2, mb, mlo, p, grid, st);
+    if (in_pairs(h, p)) {
+      // 32 value columns of the input and of its low half per CTA, 64-byte swizzle
+      using P = Cfg<false, TC_FWD, true, true>;
+      CUtensorMap mv, mo, mol;
+      if (!make_map3(&mv, A, false, TILE_COLS, fin, nt, TILE_PTS / 2, C::BKE, CU_TENSOR_MAP_SWIZZLE_64B) ||
+          !make_map3(&mlo, Alo, false, TILE_PTS, fin, nt, TILE_PTS / 2, C::BKE, CU_TENSOR_MAP_SWIZZLE_64B))
+        return map_err(h, "paired forward value rows");
+      mol = mlo;
+      if (!make_map3(&mo, e.out, false, TILE_COLS, fout, nt, TILE_PTS, BM) ||
+          (e.alo_out && !make_map3(&mol, e.alo_out, false, TILE_PTS, fout, nt, TILE_PTS, BM)))
+        return map_err(h, "paired forward outputs");
+      static bool attr_set = false;
+      pinn_status s = reserve_smem(h, k_tc_fwd_pair, P::SMEM, attr_set, "paired forward kernel");
+      if (s) return s;
+      k_tc_fwd_pair<<<grid & ~1, P::NTHREADS, P::SMEM, st>>>(ma, ma2, mb, mlo, mv, mo, mol, p);
+      return launch_check(h, "paired forward");
+    }
+  }
   return launch<TF32, TC_FWD, true>(h, ma, ma2, mb, mlo, p, grid, st);
 }
 

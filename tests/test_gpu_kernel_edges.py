@@ -113,14 +113,44 @@ def test_fused_forward_edges(cuda_lib, widths, ff, n_res):
     (PDE_MAXWELL, [40, 1024, 16], 0),         # one m-tile below a wide layer, K of 16 chunks
 ])
 @pytest.mark.parametrize("n_res", [1, 7000])  # one tile, and more units than two rounds of every SM
-def test_wide_layer_edges(cuda_lib, pde, widths, ff, n_res):
+@pytest.mark.parametrize("value_split", [False, True])
+def test_wide_layer_edges(cuda_lib, pde, widths, ff, n_res, value_split):
     """The per-layer forward and the staged adjoint of layers above 256 wide against the oracle:
     total loss and whole gradient (the residual of a single point may cancel below the
     precision's tolerance)."""
     spec = NetSpec(pde, 3 if pde == PDE_MAXWELL else 2, 1 if pde == PDE_BURGERS else 3, widths, ff_m=ff, ff_sigma=1.0)
     p, B, prob = init_params(spec, 95, 0.2), ff_matrix(spec, 96), Problem(0.02, 0.3, 2.0, 5.0)
     b = make_batch(pde, n_res, 30, 20, 97, 98)
-    gt, gg = run_gpu(spec, p, B, b, prob, "bf16")
+    gt, gg = run_gpu(spec, p, B, b, prob, "bf16", value_split=value_split)
     rt, rg = run_oracle(spec, p, B, b, prob, chunk=4096)
     assert abs(gt[0] - rt[0]) <= TOL["bf16"] * abs(rt[0])
     assert np.linalg.norm(gg - rg) <= TOL["bf16"] * np.linalg.norm(rg)
+
+
+@pytest.mark.parametrize("widths,ff", [
+    ([512, 256, 264], 0),             # layers of four and two m-tiles (in pairs), then three (not)
+    ([200, 1024, 136], 24),           # two m-tiles with a ragged second one, eight, K tails
+])
+@pytest.mark.parametrize("n_res", [1, 7000])
+def test_paired_forward_edges(cuda_lib, widths, ff, n_res):
+    """The forward in pairs of CTAs gives bitwise the loss and gradient of the unpaired launches
+    (which the grouped many-network step runs)."""
+    from paper_2604_15645_gb300 import api
+    spec = NetSpec(PDE_MAXWELL, 3, 3, widths, ff_m=ff, ff_sigma=1.0, rwf=True)
+    p, B = init_params(spec, 91, 0.2), ff_matrix(spec, 92)
+    db = api.DeviceBatch.from_host(make_batch(PDE_MAXWELL, n_res, 30, 20, 93, 94))
+    Bd = None if B is None else torch.tensor(B, device="cuda")
+    res = []
+    for grouped in (False, True):
+        multi = api.PinnMulti([spec], "bf16")
+        if Bd is not None:
+            api._lib.check_multi(api._lib.load().pinn_multi_set_ff_matrix(multi.h, 0, Bd.data_ptr()), multi.h)
+        multi.set_inputs([db], [api.make_problem(0.02)])
+        multi.grouped = grouped
+        q = torch.tensor(p, device="cuda")
+        grad, m, v = (torch.zeros_like(q) for _ in range(3))
+        loss = multi.train_step(q, grad, m, v, step=1)
+        torch.cuda.synchronize()
+        assert multi.status_poll() == 0
+        res.append((loss[0].clone(), grad))
+    assert torch.equal(res[0][0], res[1][0]) and torch.equal(res[0][1], res[1][1])
