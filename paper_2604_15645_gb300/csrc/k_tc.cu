@@ -234,9 +234,9 @@ __device__ __forceinline__ void adj_pairs8(float (&v)[4][N], int first, const ui
 // (a: points 0-15, b: 16-31).  After the swap within lane pairs, one access of the even
 // lane and one of the odd lane cover 64 consecutive bytes: a and b are the sectors
 // 16 (lane & 1) of the pair's even and of its odd feature.  (Its own inverse: loads swap back.)
-// Every 128-byte line that an instruction touches takes a cycle of the data path that shared
-// memory, the MMAs' operand reads and the bulk copies share, and that path bounds the wide
-// kernels: 16 lines per instruction instead of 32.
+// Every 128-byte line that an instruction touches takes a cycle of the L1 data path, which
+// shared memory uses too: 16 lines per instruction instead of 32.  (Maxwell 5x512 forward
+// launches 3.53 -> 3.40 ms.)
 __device__ __forceinline__ void pair_swap(uint32_t (&a)[8], uint32_t (&b)[8]) {
   const bool odd = threadIdx.x & 1;
 #pragma unroll
@@ -609,15 +609,12 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA, const CUte
     // pc + 64 r (jet row r), so every thread holds whole points of its feature.  A unit
     // row is one full 32-byte sector (16 BF16 or 8 FP32 values): partial-sector stores
     // would make L2 fetch the sector first.  FP32 units are small enough to double-buffer
-    // the TMEM loads; in the adjoint the next unit's Z rows are always loaded one unit
-    // ahead (the layer-below activations the adjoint is written in).
-    constexpr bool FAST = !TF32;
+    // the TMEM loads.
     constexpr int PARTS = EPI_WARPS / 4;                 // warps per lane quadrant
     constexpr int UPTS = TF32 ? 8 : 16;                  // points per unit
     constexpr int UNITS = TILE_PTS / (UPTS * PARTS);     // units per warp and tile
     constexpr bool PIPE = TF32;                          // double-buffered TMEM loads
     static_assert(PARTS * UNITS * UPTS == TILE_PTS && UNITS % 2 == 0, "epilogue units cover a 64-point tile");
-    constexpr int ZW = (int)sizeof(T) * UPTS / 4;        // 32-bit words of one Z row of a unit
     const int quad = warp & 3;
     const int part = (warp - 2) >> 2;
     const int row = quad * 32 + lane;
@@ -626,23 +623,28 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA, const CUte
     // BF16 tanh forward: both units of a warp's tile are finished before their sectors are exchanged
     // and stored; the accumulator is free as soon as it is in registers.
     constexpr bool PAIRS = !TF32 && !SINE && MODE == TC_FWD;
-    constexpr int ZR = 4;                                // jet rows loaded per unit
-    uint32_t znext[ZR][ZW];                              // adjoint: A rows of the next unit
-    auto load_z = [&](int t_, int u_) {
+    // TF32 forward and adjoint: two units at a time, whose sectors lane pairs exchange; the
+    // adjoint's activations of the next two units are loaded the same way before this
+    // two's stores.  (One unit at a time, a line per lane: 6x256 cavity at 69,632 points, five
+    // adjoint launches 1.71 -> 1.43 ms, six forward launches 1.29 -> 1.16.)
+    constexpr bool PAIRS32 = TF32 && !SINE && (MODE == TC_FWD || MODE == TC_ADJ);
+    [[maybe_unused]] uint32_t aw[PAIRS32 && MODE == TC_ADJ ? 2 : 1][4][8];
+    [[maybe_unused]] auto load_pairs32 = [&](int t_, int u_) {
       int mb_, nb_, k0_, k1_;
       coords(t_, mb_, nb_, k0_, k1_);
       const int m_ = mb_ * BM + row;
       if (m_ < p.M) {
-        const T* zr = reinterpret_cast<const T*>(p.e.ain) + toff(m_, (int64_t)nb_ * BN, p.M) + unit_col(u_);
+        const float* z = reinterpret_cast<const float*>(p.e.ain) + toff(m_ & ~1, (int64_t)nb_ * BN, p.M) +
+                         unit_col(u_) + UPTS * (m_ & 1);
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-          if constexpr (UPTS == 8) ld8raw(zr + 64 * r, znext[r]);
-          else ld_global_256(zr + 64 * r, znext[r]);
+          ld8raw(z + 64 * r, aw[0][r]);
+          ld8raw(z + 64 * r + TILE_COLS, aw[1][r]);
         }
       }
     };
-    if constexpr (MODE == TC_ADJ && !SINE) {
-      if (grid.bx() < total) load_z(grid.bx(), 0);
+    if constexpr (PAIRS32 && MODE == TC_ADJ) {
+      if (grid.bx() < total) load_pairs32(grid.bx(), 0);
     }
     [[maybe_unused]] int ob = 0;                          // pair: the next output buffer, its uses' parity
     [[maybe_unused]] uint32_t oph = 0;
@@ -673,79 +675,57 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA, const CUte
         }
       };
       // the epilogue of one unit of a valid row
-      auto finish = [&](int u, float (&v)[4][UPTS], const uint32_t (&zw)[ZR][ZW]) {
+      auto finish = [&](int u, float (&v)[4][UPTS]) {
         const int pc = unit_col(u);                                   // first point of the unit in its tile
         const int64_t cbase = toff(m, (int64_t)nb * BN, p.M) + pc;    // tile nb, row m
-        if constexpr (MODE == TC_FWD) {
+        if constexpr (MODE == TC_FWD && SINE) {
           const float bias = p.e.bias[m];
 #pragma unroll
           for (int i = 0; i < UPTS; ++i) v[0][i] += bias;
-          if constexpr (SINE) {
-            // the pre-activation jets for the adjoint, FP32 [M][NC] tile-major
-            float* zo = p.e.zout + cbase;
+          // the pre-activation jets for the adjoint, FP32 [M][NC] tile-major
+          float* zo = p.e.zout + cbase;
 #pragma unroll
-            for (int r = 0; r < 4; ++r) st_f32<UPTS>(zo + 64 * r, v[r]);
-          }
+          for (int r = 0; r < 4; ++r) st_f32<UPTS>(zo + 64 * r, v[r]);
 #pragma unroll
           for (int i = 0; i < UPTS; ++i) {
             float z[4] = {v[0][i], v[1][i], v[2][i], v[3][i]}, a[4];
-            if constexpr (SINE) jet_fwd_sine(z, a, p.e.jet_mode, p.e.omega0);
-            else jet_fwd<FAST>(z, a, p.e.jet_mode);
+            jet_fwd_sine(z, a, p.e.jet_mode, p.e.omega0);
 #pragma unroll
             for (int r = 0; r < 4; ++r) v[r][i] = a[r];
           }
           T* ao = reinterpret_cast<T*>(p.e.out) + cbase;
 #pragma unroll
           for (int r = 0; r < 4; ++r) st_row(ao + 64 * r, v[r]);
-          if constexpr (TF32) {
-            if (p.e.out_pm) store_pm8(reinterpret_cast<float*>(p.e.out_pm), (int64_t)nb * BN + pc, p.M, m, v);
-          }
-          if (!TF32 && p.e.alo_out) {
+          if (p.e.alo_out) {
             // low half of the value rows for the next forward (BF16 rounding remainder)
             float lo[UPTS];
 #pragma unroll
             for (int i = 0; i < UPTS; ++i) lo[i] = v[0][i] - __bfloat162float(__float2bfloat16_rn(v[0][i]));
             st_row(reinterpret_cast<T*>(p.e.alo_out) + loff(m, (int64_t)nb * TILE_PTS, p.M) + pc, lo);
           }
-        } else if constexpr (MODE == TC_ADJ) {
-          if constexpr (SINE) {
-            // the rule from the stored pre-activation jets z of the layer below
-            const float* zr = p.e.zin + cbase;
+        } else if constexpr (MODE == TC_ADJ && SINE) {
+          // the rule from the stored pre-activation jets z of the layer below
+          const float* zr = p.e.zin + cbase;
 #pragma unroll
-            for (int h8 = 0; h8 < UPTS / 8; ++h8) {
-              uint32_t zz[4][8];
+          for (int h8 = 0; h8 < UPTS / 8; ++h8) {
+            uint32_t zz[4][8];
 #pragma unroll
-              for (int r = 0; r < 4; ++r) ld_global_256(zr + 64 * r + 8 * h8, zz[r]);
+            for (int r = 0; r < 4; ++r) ld_global_256(zr + 64 * r + 8 * h8, zz[r]);
 #pragma unroll
-              for (int i = 0; i < 8; ++i) {
-                float z[4] = {__uint_as_float(zz[0][i]), __uint_as_float(zz[1][i]), __uint_as_float(zz[2][i]),
-                              __uint_as_float(zz[3][i])};
-                const int k = 8 * h8 + i;
-                float ab[4] = {v[0][k], v[1][k], v[2][k], v[3][k]}, zb[4];
-                jet_adj_sine(z, ab, zb, p.e.jet_mode, p.e.omega0);
+            for (int i = 0; i < 8; ++i) {
+              float z[4] = {__uint_as_float(zz[0][i]), __uint_as_float(zz[1][i]), __uint_as_float(zz[2][i]),
+                            __uint_as_float(zz[3][i])};
+              const int k = 8 * h8 + i;
+              float ab[4] = {v[0][k], v[1][k], v[2][k], v[3][k]}, zb[4];
+              jet_adj_sine(z, ab, zb, p.e.jet_mode, p.e.omega0);
 #pragma unroll
-                for (int r = 0; r < 4; ++r) v[r][k] = zb[r];
-              }
-            }
-          } else {
-#pragma unroll
-            for (int i = 0; i < UPTS; ++i) {
-              float av[4];
-#pragma unroll
-              for (int r = 0; r < 4; ++r) av[r] = raw_elem<T>(zw[r], i);
-              float ab[4] = {v[0][i], v[1][i], v[2][i], v[3][i]}, zb[4];
-              jet_adj_a(av, ab, zb, p.e.jet_mode);
-#pragma unroll
-              for (int r = 0; r < 4; ++r) v[r][i] = zb[r];
+              for (int r = 0; r < 4; ++r) v[r][k] = zb[r];
             }
           }
           if (p.e.out) {
             T* zbo = reinterpret_cast<T*>(p.e.out) + cbase;
 #pragma unroll
             for (int r = 0; r < 4; ++r) st_row(zbo + 64 * r, v[r]);
-          }
-          if constexpr (TF32) {
-            if (p.e.out_pm) store_pm8(reinterpret_cast<float*>(p.e.out_pm), (int64_t)nb * BN + pc, p.M, m, v);
           }
         } else if constexpr (MODE == TC_DW) {
           const int split = t / (p.m_tiles * p.n_tiles);
@@ -760,30 +740,23 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA, const CUte
                 if (col0 + j < p.N) dst[col0 + j] = v[r][j];
             }
           }
-        } else {   // TC_STORE
+        } else if constexpr (MODE == TC_STORE) {
 #pragma unroll
           for (int r = 0; r < 4; ++r) st_f32<UPTS>(p.out32 + cbase + 64 * r, v[r]);
         }
       };
-      auto process = [&](int u, float (&v)[4][UPTS]) {
-        uint32_t zw[ZR][ZW];
-        if constexpr (MODE == TC_ADJ && !SINE) {
+      // bias gradient of the layer below (value rows) and, for a first layer on raw
+      // coordinates, the coordinate terms of its weight gradient (every lane: rows past M
+      // add values that nobody stores)
+      [[maybe_unused]] auto bias_sums = [&](int u, const float (&v)[4][UPTS]) {
+        if (!p.e.dbpart) return;
 #pragma unroll
-          for (int r = 0; r < ZR; ++r)
-#pragma unroll
-            for (int j = 0; j < ZW; ++j) zw[r][j] = znext[r][j];
-          if (u + 1 < UNITS) load_z(t, u + 1);
-          else if (t + grid.gdim() < total) load_z(t + grid.gdim(), 0);
-        }
-        if (mvalid) finish(u, v, zw);
-        if (MODE == TC_ADJ && p.e.dbpart) {
-          // bias gradient of the layer below (value rows) and, for a first layer on raw
-          // coordinates, the coordinate terms of its weight gradient (every lane: rows past M
-          // add values that nobody stores)
-#pragma unroll
-          for (int i = 0; i < UPTS; ++i) db[0] += v[0][i];
-          if (p.e.dterms) coord_terms<UPTS>(v, xc, UPTS * u, p.e.dterms, p.e.jet_mode, db);
-        }
+        for (int i = 0; i < UPTS; ++i) db[0] += v[0][i];
+        if (p.e.dterms) coord_terms<UPTS>(v, xc, UPTS * u, p.e.dterms, p.e.jet_mode, db);
+      };
+      [[maybe_unused]] auto process = [&](int u, float (&v)[4][UPTS]) {
+        if (mvalid) finish(u, v);
+        if constexpr (MODE == TC_ADJ) bias_sums(u, v);
       };
 
       if constexpr (PAIRS) {
@@ -832,6 +805,64 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA, const CUte
           store_pairs(reinterpret_cast<T*>(p.e.out), w, m, nb, p.M, unit_col(0));
           if (p.e.alo_out) store_lo_pairs(reinterpret_cast<T*>(p.e.alo_out), lo, m, nb, p.M, unit_col(0));
         }
+      } else if constexpr (PAIRS32) {
+        [[maybe_unused]] const float bias = MODE == TC_FWD && mvalid ? p.e.bias[m] : 0.f;
+#pragma unroll 1
+        for (int u = 0; u < UNITS; u += 2) {
+          float v[2][4][UPTS];
+          issue(u, v[0]);
+          issue(u + 1, v[1]);
+          tmem_wait_ld();
+          if (u + 2 == UNITS) {
+            tc_fence_before();
+            mbar_arrive(&acc_empty[buf]);
+          }
+          if constexpr (MODE == TC_ADJ) {
+#pragma unroll
+            for (int r = 0; r < 4; ++r) pair_swap(aw[0][r], aw[1][r]);
+          }
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+#pragma unroll
+            for (int i = 0; i < UPTS; ++i) {
+              float y[4];
+              if constexpr (MODE == TC_FWD) {
+                const float z[4] = {v[k][0][i] + bias, v[k][1][i], v[k][2][i], v[k][3][i]};
+                jet_fwd<false>(z, y, p.e.jet_mode);
+              } else {
+                const float ab[4] = {v[k][0][i], v[k][1][i], v[k][2][i], v[k][3][i]};
+                const float av[4] = {__uint_as_float(aw[k][0][i]), __uint_as_float(aw[k][1][i]),
+                                     __uint_as_float(aw[k][2][i]), __uint_as_float(aw[k][3][i])};
+                jet_adj_a(av, ab, y, p.e.jet_mode);
+              }
+#pragma unroll
+              for (int r = 0; r < 4; ++r) v[k][r][i] = y[r];
+            }
+            if constexpr (MODE == TC_ADJ) bias_sums(u + k, v[k]);
+          }
+          if constexpr (MODE == TC_ADJ) {
+            if (u + 2 < UNITS) load_pairs32(t, u + 2);
+            else if (t + grid.gdim() < total) load_pairs32(t + grid.gdim(), 0);
+          }
+          if (p.e.out_pm && mvalid) {
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+              store_pm8(reinterpret_cast<float*>(p.e.out_pm), (int64_t)nb * BN + unit_col(u + k), p.M, m, v[k]);
+          }
+          if (p.e.out) {
+            float* o = reinterpret_cast<float*>(p.e.out) + toff(m & ~1, (int64_t)nb * BN, p.M) + unit_col(u) + UPTS * (m & 1);
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+              uint32_t (&x)[8] = reinterpret_cast<uint32_t (&)[8]>(v[0][r]);
+              uint32_t (&y)[8] = reinterpret_cast<uint32_t (&)[8]>(v[1][r]);
+              pair_swap(x, y);
+              if (mvalid) {
+                st_global_256(o + 64 * r, x);
+                st_global_256(o + 64 * r + TILE_COLS, y);
+              }
+            }
+          }
+        }
       } else if constexpr (PIPE) {
         float va[4][UPTS], vb[4][UPTS];
         issue(0, va);
@@ -862,7 +893,7 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA, const CUte
           if (j < p.e.dterms) dst[1 + j] = db[1 + j];
       }
       }   // half
-      if constexpr (!PAIRS) {
+      if constexpr (!PAIRS && !PAIRS32) {
         tc_fence_before();
         mbar_arrive(&acc_empty[buf]);
       }
@@ -897,15 +928,16 @@ __global__ void __launch_bounds__(Cfg<TF32, MODE, SPLIT>::NTHREADS, 1)
   tc_gemm_body<TF32, MODE, SPLIT, SINE>(&mapA, &mapA2, &mapB, &mapBlo, p, SingleGrid{});
 }
 
-// The BF16 tanh forward in pairs.  Launched alone, a 128 x 256 unit of a 512-wide layer is
-// bound by the path of shared memory: 24 KB of operands per K step and 72 KB of copies per
-// stage, a cycle per 128 bytes.  As a pair each CTA stages half of the columns (56 KB) and its
-// MMAs read half of them (18 KB); the smaller stages leave room for output buffers, from which
-// the tile leaves by bulk tensor stores.  Same sums in the same order.  Forward launches,
-// ms: Maxwell 5x512 at 294,912 points 3.38 -> 3.09, 8x512 cavity at 1,064,960 23.4 -> 22.2.
-// (Pairs that store from registers: 3.28 and 24.3.)  What bounds it now: neither the MMAs (no
-// faster with the low half of the weights on the value rows only) nor HBM (57%); without its
-// epilogue the unpaired kernel took 0.71 of its time.
+// The BF16 tanh forward in pairs.  Launched alone, a 128 x 256 unit of a 512-wide layer moves
+// 24 KB of operands per K step and 72 KB of copies per stage through shared memory and stores
+// a line per lane; at 128 bytes a cycle the sum (13,300 cycles) is its time (13,450).  As a
+// pair each CTA stages half of the columns (56 KB) and its MMAs read half of them (18 KB); the
+// smaller stages leave room for output buffers, from which the tile leaves by bulk tensor
+// stores.  Same sums in the same order.  Forward launches, ms: Maxwell 5x512 at 294,912
+// points 3.38 -> 3.09, 8x512 cavity at 1,064,960 23.4 -> 22.2.  (Pairs that store from
+// registers: 3.28 and 24.3.)  Left: tensor pipe 53%, DRAM 45%; limiting the low half of the
+// weights to the value rows saves nothing, and without its epilogue the unpaired kernel took
+// 0.71 of its time.
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Cfg<false, TC_FWD, true, true>::NTHREADS, 1)
     k_tc_fwd_pair(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapA2,
                   const __grid_constant__ CUtensorMap mapB, const __grid_constant__ CUtensorMap mapBlo,
@@ -1259,8 +1291,9 @@ pinn_status tc_gemm_dw(pinn_handle* h, const void* Zbar, const void* A, int fout
 // once: the separate weight-gradient pass and its re-reads are gone.
 // The epilogue works on packed pairs of points, and the next unit's Zbar is prefetched into
 // L2: five launches of the 6x256 cavity at 69,632 points 0.497 -> 0.471 ms.  What bounds it
-// now: the path of shared memory, which the MMAs' operands (N = 64: 6 KB per 32 cycles),
-// the bulk copies and the stores share.
+// now: no single unit (DRAM 56%, tensor pipe 37%, L1/shared memory 43%), but the time a stage
+// takes to arrive: two stages of 48 KB, 3,400 cycles each under this traffic (without the
+// stores 0.39 ms, with every load in L2 0.41).
 //
 // DW = false is the adjoint alone, for a layer whose fan-out is above 256 (its dW^T slab
 // would fill tensor memory).  Two accumulators overlap the epilogue with the next unit's MMAs;

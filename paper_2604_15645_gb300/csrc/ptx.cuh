@@ -247,14 +247,5 @@ __device__ __forceinline__ void st_f32(float* p, const float* v) {
   for (int i = 0; i < N; i += 8) st_global_256(p + i, reinterpret_cast<const uint32_t*>(v + i));
 }
 __device__ __forceinline__ void ld8raw(const float* p, uint32_t w[8]) { ld_global_256(p, w); }
-// Element i of 8 raw row words (BF16 pairs or FP32).
-template <typename T>
-__device__ __forceinline__ float raw_elem(const uint32_t* w, int i) {
-  if (sizeof(T) == 2) {
-    const uint32_t x = w[i >> 1];
-    return __uint_as_float((i & 1) ? (x & 0xFFFF0000u) : (x << 16));
-  }
-  return __uint_as_float(w[i]);
-}
 
 }  // namespace pinn

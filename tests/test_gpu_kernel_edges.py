@@ -154,3 +154,20 @@ def test_paired_forward_edges(cuda_lib, widths, ff, n_res):
         assert multi.status_poll() == 0
         res.append((loss[0].clone(), grad))
     assert torch.equal(res[0][0], res[1][0]) and torch.equal(res[0][1], res[1][1])
+
+
+@pytest.mark.parametrize("pde,widths,ff", [
+    (PDE_NS, [136, 24, 200], 8),      # ragged m-tiles and K blocks
+    (PDE_BURGERS, [72, 264], 0),      # raw first layer (coordinate terms), three m-tiles
+])
+@pytest.mark.parametrize("n_res", [1, 7000])
+def test_tf32_edges(cuda_lib, pde, widths, ff, n_res):
+    """The TF32 epilogues against the oracle.  Bound: the weight gradient truncates both operands
+    to 10 mantissa bits, at most 2^-10 of each."""
+    spec = NetSpec(pde, 2, 1 if pde == PDE_BURGERS else 3, widths, ff_m=ff, ff_sigma=1.0)
+    p, B, prob = init_params(spec, 81, 0.2), ff_matrix(spec, 82), Problem(0.02, 0.3, 2.0, 5.0)
+    b = make_batch(pde, n_res, 30, 20, 83, 84)
+    gt, gg = run_gpu(spec, p, B, b, prob, "tf32")
+    rt, rg = run_oracle(spec, p, B, b, prob, chunk=4096)
+    assert abs(gt[0] - rt[0]) <= TOL["tf32"] * abs(rt[0])
+    assert np.linalg.norm(gg - rg) <= 2.0 ** -9 * np.linalg.norm(rg)
