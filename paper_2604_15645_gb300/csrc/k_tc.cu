@@ -19,12 +19,14 @@
 // layer before) and add both truncation remainders: W_hi B + W_lo B + W_hi B_lo, with
 // B_lo = B - tf32(B) computed in shared memory by two converter warps.
 //
-// Warp roles per CTA (320 threads, 384 with converters, one CTA per SM, persistent):
+// Warp roles per CTA (320 threads, 384 with converters, 352 in pairs, one CTA per SM,
+// persistent):
 //   warp 0     TMA producer (one lane)
 //   warp 1     TMEM allocator + MMA issuer (one lane)
 //   warps 2-9  epilogue; warp w reads TMEM lanes 32*(w%4) .. +31 and handles the
 //              points 32*((w-2)/4) .. +31 of the tile, 16 at a time
 //   warps 10-11 (TF32 forward / adjoint only) B_lo converters
+//   warp 10    (pairs only) output stores
 // Two accumulator buffers of 256 columns let the epilogue of one tile overlap the
 // MMAs of the next.  Every mbarrier wait is bounded (global timer); on expiry the
 // CTA latches PINN_ERR_TIMEOUT in the status word, stops issuing work, waits for
