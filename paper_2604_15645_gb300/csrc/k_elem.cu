@@ -1638,8 +1638,9 @@ cudaError_t launch_out_loss_mma(const OutArgs& a, int nblocks, cudaStream_t st) 
 template <typename T, int D, bool FAST, bool SINE>
 cudaError_t out_loss_launch(const OutArgs& a, int nblocks, size_t smem, cudaStream_t st) {
   auto kern = k_out_loss<T, D, FAST, SINE>;
-  // weights + per-warp dW accumulators: up to 120 KB for 2048-wide, 3-output networks
-  static size_t reserved = 48 * 1024;
+  // weights + per-warp dW accumulators: up to 152 KB for 2048-wide, 3-output networks.  (Asked
+  // for from the first byte: the 48 KB that need no asking hold the static memory as well.)
+  static size_t reserved = 0;
   if (smem > reserved) {
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
