@@ -59,6 +59,21 @@ int pde_dout(int pde) { return (pde == PINN_NS_STEADY_2D || pde == PINN_MAXWELL_
 
 namespace pinn {
 
+cudaError_t allow_smem(pinn_handle* h, const void* kern, size_t bytes) {
+  return h->smem.allow(kern, bytes, cudaSuccess, cudaErrorInvalidValue, [&](size_t* limit) {
+    cudaFuncAttributes fa;
+    int optin = 0;
+    cudaError_t e = cudaFuncGetAttributes(&fa, kern);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
+    if (e == cudaSuccess) {
+      *limit = (size_t)optin - fa.sharedSizeBytes;
+      e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*limit);
+    }
+    if (e != cudaSuccess) cudaGetLastError();   // do not leave the failure for the next launch to report
+    return e;
+  });
+}
+
 pinn_status make_plan(const pinn_handle* h, int64_t n_res, int64_t n_ic, int64_t n_bc, Plan* p) {
   Plan q;
   q.n_res = n_res; q.n_ic = n_ic; q.n_bc = n_bc;
@@ -314,9 +329,8 @@ struct Pass {
     if (cp.tc[li])
       return tc_gemm_fwd(h, ws + cp.lay[li].wc, ws + cp.lay[li].wlo, ws + p.A[li], ws + p.Alo[li], cp.lay[li].fout,
                          cp.lay[li].fin, p.NC, e, st);
-    launch_simt_gemm_fwd(W32(li), WT32(li), ws + p.A[li], cp.lay[li].fout, cp.lay[li].fin, p.NP, e, prec, h->sm_count,
-                         st);
-    return PINN_OK;
+    return cuda_check(h, launch_simt_gemm_fwd(h, W32(li), WT32(li), ws + p.A[li], cp.lay[li].fout, cp.lay[li].fin, p.NP,
+                                              e, prec, st), "CUDA-core forward launch");
   }
 
   // 4-5 for loss term t (one weighted term, or term t of the per-term gradients):
@@ -369,7 +383,7 @@ struct Pass {
         o1.want_grad = 0;
         o1.segpart = reinterpret_cast<double*>(ws + p.segpart);
         PhaseScope ps(h, st, PH_OUT, 1);
-        const cudaError_t e = launch_out_loss(o1, prec, p.nloss_blocks, st);
+        const cudaError_t e = launch_out_loss(h, o1, prec, p.nloss_blocks, st);
         if (e != cudaSuccess) return cuda_check(h, e, "output/loss launch");
         launch_finalize_causal(o1.segpart, o1.losspart, p.nloss_blocks, h->causal_M, h->causal_eps,
                                b->ic_mask ? pc.N_ic : 0, b->bc_mask ? pc.N_bc : 0, prob->lambda_pde,
@@ -380,7 +394,7 @@ struct Pass {
     }
     if (!causal || want_grad) {
       PhaseScope ps(h, st, PH_OUT, 1);
-      const cudaError_t e = launch_out_loss(oa, prec, p.nloss_blocks, st);
+      const cudaError_t e = launch_out_loss(h, oa, prec, p.nloss_blocks, st);
       if (e != cudaSuccess) return cuda_check(h, e, "output/loss launch");
     }
     if (term == 0 && !causal) {   // the loss terms are unweighted sums; the total uses the problem's weights
@@ -421,8 +435,10 @@ struct Pass {
                        st);
         if (s) return s;
       } else {
-        launch_simt_gemm_dw(zb, ws + p.A[li], lp.fout, lp.fin, p.NC, lp.nsplit, reinterpret_cast<float*>(ws + lp.dwpart),
-                            prec, st);
+        s = cuda_check(h, launch_simt_gemm_dw(h, zb, ws + p.A[li], lp.fout, lp.fin, p.NC, lp.nsplit,
+                                              reinterpret_cast<float*>(ws + lp.dwpart), prec, st),
+                       "CUDA-core weight-gradient launch");
+        if (s) return s;
       }
     }
     if (!cp.fused_db[li] && !(li == L - 1 && cp.out_db)) {
@@ -435,7 +451,9 @@ struct Pass {
       // its contraction with the embedding's derivatives by B (or the periods).
       PhaseScope ps(h, st, PH_OTHER, 3);
       double* ffpart = reinterpret_cast<double*>(ws + p.ffpart);
-      launch_simt_gemm_lin(WT32(li), W32(li), zb, lp.fin, lp.fout, p.NP, ws + p.Zbar[0], prec, h->sm_count, st);
+      s = cuda_check(h, launch_simt_gemm_lin(h, WT32(li), W32(li), zb, lp.fin, lp.fout, p.NP, ws + p.Zbar[0], prec, st),
+                     "input-jet adjoint launch");
+      if (s) return s;
       launch_ff_grad(ws + p.Zbar[0], b->x_res, b->x_ic, b->x_bc, p.n_res, p.n_ic, p.n_bc, h->d_in, h->ff_B,
                      h->spec.ff_m, mode, p.NP, ffpart, prec, st);
       launch_ff_grad_final(ffpart, h->d_in, h->spec.ff_m, h->periodic, h->periods, pc.first ? 0 : 1, d_grad_ff, st);
@@ -468,8 +486,8 @@ struct Pass {
       return tc_gemm_adj(h, ws + lp.wtc, ws + lp.wtlo, ws + cp.zbpm[(li + 1) % 2], lp.fin, lp.fout, p.NC, e, st);
     }
     if (cp.tc[li]) return tc_gemm_adj(h, ws + lp.wtc, nullptr, zb, lp.fin, lp.fout, p.NC, e, st);
-    launch_simt_gemm_adj(WT32(li), W32(li), zb, lp.fin, lp.fout, p.NP, e, prec, h->sm_count, st);
-    return PINN_OK;
+    return cuda_check(h, launch_simt_gemm_adj(h, WT32(li), W32(li), zb, lp.fin, lp.fout, p.NP, e, prec, st),
+                      "CUDA-core adjoint launch");
   }
 
   // 7. Ordered FP64 reduction + RWF chain rule into the packed gradient.

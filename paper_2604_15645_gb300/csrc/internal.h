@@ -7,6 +7,7 @@
 #include <cuda_bf16.h>
 
 #include "../../include/pinn.h"
+#include "smem_limit.h"
 
 namespace pinn {
 
@@ -80,6 +81,7 @@ struct pinn_graph_key {
 
 struct pinn_handle {
   pinn_spec spec{};
+  pinn::SmemLimits smem;     // kernels whose shared-memory limit has been raised for this handle
   int d_in = 0, d_out = 0, L = 0;
   int jet_mode = 0;
   int first_gemm = 0;        // index of the first hidden layer computed by a GEMM (0 with FF, 1 without)
@@ -118,6 +120,9 @@ struct pinn_handle {
 };
 
 namespace pinn {
+
+// Before a launch of `kern` with `bytes` of dynamic shared memory (see smem_limit.h).
+cudaError_t allow_smem(pinn_handle* h, const void* kern, size_t bytes);
 
 pinn_status make_plan(const pinn_handle* h, int64_t n_res, int64_t n_ic, int64_t n_bc, Plan* plan);
 
@@ -168,19 +173,19 @@ struct EpiArgs {
 
 // CUDA-core GEMMs: D[M][4 NP] = A[M][K] Bop[K][4 NP] (+ epilogue), Bop the jets in the
 // compute type.  The FP32 weights are given in both orientations, [fout][fin] (W) and
-// [fin][fout] (WT); sms is the device's SM count.
+// [fin][fout] (WT).  They return what the launch returned.
 //   forward  A = W   (M = fout, K = fin)
 //   adjoint  A = W^T (M = fin, K = fout)
 //   lin      A = W^T with no epilogue (the input-jet adjoint W_1^T Zbar_1)
-void launch_simt_gemm_fwd(const float* W, const float* WT, const void* Bop, int M, int K, int64_t NP, const EpiArgs& e,
-                          int prec, int sms, cudaStream_t st);
-void launch_simt_gemm_adj(const float* WT, const float* W, const void* Bop, int M, int K, int64_t NP, const EpiArgs& e,
-                          int prec, int sms, cudaStream_t st);
-void launch_simt_gemm_lin(const float* WT, const float* W, const void* Bop, int M, int K, int64_t NP, void* out,
-                          int prec, int sms, cudaStream_t st);
+cudaError_t launch_simt_gemm_fwd(pinn_handle* h, const float* W, const float* WT, const void* Bop, int M, int K,
+                                 int64_t NP, const EpiArgs& e, int prec, cudaStream_t st);
+cudaError_t launch_simt_gemm_adj(pinn_handle* h, const float* WT, const float* W, const void* Bop, int M, int K,
+                                 int64_t NP, const EpiArgs& e, int prec, cudaStream_t st);
+cudaError_t launch_simt_gemm_lin(pinn_handle* h, const float* WT, const float* W, const void* Bop, int M, int K,
+                                 int64_t NP, void* out, int prec, cudaStream_t st);
 // part[s][M][N] = sum_{k in split s} Aop[m][k] Bop[n][k], both in the compute type, tile-major.
-void launch_simt_gemm_dw(const void* Aop, const void* Bop, int M, int N, int64_t NC, int nsplit, float* part, int prec,
-                         cudaStream_t st);
+cudaError_t launch_simt_gemm_dw(pinn_handle* h, const void* Aop, const void* Bop, int M, int N, int64_t NC, int nsplit,
+                                float* part, int prec, cudaStream_t st);
 
 struct OutArgs {
   const void* AL;        // A_L^T [w][NC] compute type
@@ -223,7 +228,7 @@ void launch_ff_grad(const void* Abar0, const float* x_res, const float* x_ic, co
                     double* part, int prec, cudaStream_t st);
 void launch_ff_grad_final(const double* part, int d_in, int m, bool periodic, const double* periods, int accumulate,
                           float* out, cudaStream_t st);
-cudaError_t launch_out_loss(const OutArgs& a, int prec, int nblocks, cudaStream_t st);
+cudaError_t launch_out_loss(pinn_handle* h, const OutArgs& a, int prec, int nblocks, cudaStream_t st);
 int out_loss_blocks(int64_t n_points);
 // The output/loss kernel with A_L staged by TMA (BF16 tanh networks, last hidden width
 // <= 512) runs two blocks per SM; its block count (the number of loss, dW and bias

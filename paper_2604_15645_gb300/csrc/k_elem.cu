@@ -1043,22 +1043,18 @@ static size_t ot_smem(int w, int d_out) {
 }
 
 template <int D, int MODE, bool LO>
-cudaError_t out_loss_tma_launch(const CUtensorMap& ma, const CUtensorMap& ml, const OutArgs& a, int nblocks,
-                                cudaStream_t st) {
+cudaError_t out_loss_tma_launch(pinn_handle* h, const CUtensorMap& ma, const CUtensorMap& ml, const OutArgs& a,
+                                int nblocks, cudaStream_t st) {
   auto kern = k_out_loss_tma<D, MODE, LO>;
   const size_t smem = ot_smem(a.w, D);
-  static size_t reserved = 0;
-  if (smem > reserved) {
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    reserved = smem;
-  }
+  const cudaError_t e = allow_smem(h, reinterpret_cast<const void*>(kern), smem);
+  if (e != cudaSuccess) return e;
   kern<<<nblocks, OT_THREADS, smem, st>>>(ma, ml, a);
   return cudaGetLastError();
 }
 
 // Returns cudaErrorNotSupported (nothing launched) when the tensor maps cannot be built.
-cudaError_t launch_out_loss_tma(const OutArgs& a, int nblocks, cudaStream_t st) {
+cudaError_t launch_out_loss_tma(pinn_handle* h, const OutArgs& a, int nblocks, cudaStream_t st) {
   CUtensorMap ma, ml;
   const uint64_t nt = (uint64_t)(a.NP / TILE_PTS);
   if (!tc_map3(&ma, a.AL, false, TILE_COLS, (uint64_t)a.w, nt, 64, OT_FC)) return cudaErrorNotSupported;
@@ -1066,14 +1062,14 @@ cudaError_t launch_out_loss_tma(const OutArgs& a, int nblocks, cudaStream_t st) 
   if (a.ALlo && !tc_map3(&ml, a.ALlo, false, TILE_PTS, (uint64_t)a.w, nt, 64, OT_FC)) return cudaErrorNotSupported;
   const bool lo = a.ALlo != nullptr;
   if (a.d_out == 1 && a.jet_mode == JET_BURGERS)
-    return lo ? out_loss_tma_launch<1, JET_BURGERS, true>(ma, ml, a, nblocks, st)
-              : out_loss_tma_launch<1, JET_BURGERS, false>(ma, ml, a, nblocks, st);
+    return lo ? out_loss_tma_launch<1, JET_BURGERS, true>(h, ma, ml, a, nblocks, st)
+              : out_loss_tma_launch<1, JET_BURGERS, false>(h, ma, ml, a, nblocks, st);
   if (a.d_out == 3 && a.jet_mode == JET_NS)
-    return lo ? out_loss_tma_launch<3, JET_NS, true>(ma, ml, a, nblocks, st)
-              : out_loss_tma_launch<3, JET_NS, false>(ma, ml, a, nblocks, st);
+    return lo ? out_loss_tma_launch<3, JET_NS, true>(h, ma, ml, a, nblocks, st)
+              : out_loss_tma_launch<3, JET_NS, false>(h, ma, ml, a, nblocks, st);
   if (a.d_out == 3 && a.jet_mode == JET_MAXWELL)
-    return lo ? out_loss_tma_launch<3, JET_MAXWELL, true>(ma, ml, a, nblocks, st)
-              : out_loss_tma_launch<3, JET_MAXWELL, false>(ma, ml, a, nblocks, st);
+    return lo ? out_loss_tma_launch<3, JET_MAXWELL, true>(h, ma, ml, a, nblocks, st)
+              : out_loss_tma_launch<3, JET_MAXWELL, false>(h, ma, ml, a, nblocks, st);
   return cudaErrorNotSupported;
 }
 
@@ -1598,21 +1594,17 @@ bool out_loss_mma_ok(int prec, int act, int w) {
 }
 
 template <int D, int MODE, bool LO>
-cudaError_t out_loss_mma_launch(const CUtensorMap& ma, const CUtensorMap& ml, const CUtensorMap& mz, const OutArgs& a,
-                                int nblocks, cudaStream_t st) {
+cudaError_t out_loss_mma_launch(pinn_handle* h, const CUtensorMap& ma, const CUtensorMap& ml, const CUtensorMap& mz,
+                                const OutArgs& a, int nblocks, cudaStream_t st) {
   auto kern = k_out_loss_mma<D, MODE, LO>;
   const size_t smem = (size_t)OmLayout(a.w, D).total + 1024;
-  static size_t reserved = 0;
-  if (smem > reserved) {
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    reserved = smem;
-  }
+  const cudaError_t e = allow_smem(h, reinterpret_cast<const void*>(kern), smem);
+  if (e != cudaSuccess) return e;
   kern<<<nblocks, OT_THREADS, smem, st>>>(ma, ml, mz, a);
   return cudaGetLastError();
 }
 
-cudaError_t launch_out_loss_mma(const OutArgs& a, int nblocks, cudaStream_t st) {
+cudaError_t launch_out_loss_mma(pinn_handle* h, const OutArgs& a, int nblocks, cudaStream_t st) {
   CUtensorMap ma, ml, mz;
   const uint64_t nt = (uint64_t)(a.NP / TILE_PTS);
   if (!tc_map3(&ma, a.AL, false, TILE_COLS, (uint64_t)a.w, nt, 64, OT_FC)) return cudaErrorNotSupported;
@@ -1623,40 +1615,36 @@ cudaError_t launch_out_loss_mma(const OutArgs& a, int nblocks, cudaStream_t st) 
   if (a.ALlo && !tc_map3(&ml, a.ALlo, false, TILE_PTS, (uint64_t)a.w, nt, 64, OT_FC)) return cudaErrorNotSupported;
   const bool lo = a.ALlo != nullptr;
   if (a.d_out == 1 && a.jet_mode == JET_BURGERS)
-    return lo ? out_loss_mma_launch<1, JET_BURGERS, true>(ma, ml, mz, a, nblocks, st)
-              : out_loss_mma_launch<1, JET_BURGERS, false>(ma, ml, mz, a, nblocks, st);
+    return lo ? out_loss_mma_launch<1, JET_BURGERS, true>(h, ma, ml, mz, a, nblocks, st)
+              : out_loss_mma_launch<1, JET_BURGERS, false>(h, ma, ml, mz, a, nblocks, st);
   if (a.d_out == 3 && a.jet_mode == JET_NS)
-    return lo ? out_loss_mma_launch<3, JET_NS, true>(ma, ml, mz, a, nblocks, st)
-              : out_loss_mma_launch<3, JET_NS, false>(ma, ml, mz, a, nblocks, st);
+    return lo ? out_loss_mma_launch<3, JET_NS, true>(h, ma, ml, mz, a, nblocks, st)
+              : out_loss_mma_launch<3, JET_NS, false>(h, ma, ml, mz, a, nblocks, st);
   if (a.d_out == 3 && a.jet_mode == JET_MAXWELL)
-    return lo ? out_loss_mma_launch<3, JET_MAXWELL, true>(ma, ml, mz, a, nblocks, st)
-              : out_loss_mma_launch<3, JET_MAXWELL, false>(ma, ml, mz, a, nblocks, st);
+    return lo ? out_loss_mma_launch<3, JET_MAXWELL, true>(h, ma, ml, mz, a, nblocks, st)
+              : out_loss_mma_launch<3, JET_MAXWELL, false>(h, ma, ml, mz, a, nblocks, st);
   return cudaErrorNotSupported;
 }
 
 
 template <typename T, int D, bool FAST, bool SINE>
-cudaError_t out_loss_launch(const OutArgs& a, int nblocks, size_t smem, cudaStream_t st) {
+cudaError_t out_loss_launch(pinn_handle* h, const OutArgs& a, int nblocks, size_t smem, cudaStream_t st) {
   auto kern = k_out_loss<T, D, FAST, SINE>;
   // weights + per-warp dW accumulators: up to 152 KB for 2048-wide, 3-output networks.  (Asked
   // for from the first byte: the 48 KB that need no asking hold the static memory as well.)
-  static size_t reserved = 0;
-  if (smem > reserved) {
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    reserved = smem;
-  }
+  const cudaError_t e = allow_smem(h, reinterpret_cast<const void*>(kern), smem);
+  if (e != cudaSuccess) return e;
   kern<<<nblocks, OUT_THREADS, smem, st>>>(a);
   return cudaGetLastError();
 }
 
-cudaError_t launch_out_loss(const OutArgs& a, int prec, int nblocks, cudaStream_t st) {
+cudaError_t launch_out_loss(pinn_handle* h, const OutArgs& a, int prec, int nblocks, cudaStream_t st) {
   if (!a.ZL && out_loss_mma_ok(prec, PINN_ACT_TANH, a.w)) {
-    const cudaError_t e = launch_out_loss_mma(a, nblocks, st);
+    const cudaError_t e = launch_out_loss_mma(h, a, nblocks, st);
     if (e != cudaErrorNotSupported) return e;
   }
   if (!a.ZL && out_loss_tma_ok(prec, PINN_ACT_TANH, a.w)) {
-    const cudaError_t e = launch_out_loss_tma(a, nblocks, st);
+    const cudaError_t e = launch_out_loss_tma(h, a, nblocks, st);
     if (e != cudaErrorNotSupported) return e;
   }
   const size_t smem = sizeof(float) * a.w * (a.d_out * (1 + OUT_THREADS / 32) + OUT_THREADS / 32);
@@ -1664,16 +1652,16 @@ cudaError_t launch_out_loss(const OutArgs& a, int prec, int nblocks, cudaStream_
   // tanh kernels carry none of its registers
   if (a.ZL) {
     if (prec == PINN_BF16)
-      return a.d_out == 1 ? out_loss_launch<__nv_bfloat16, 1, true, true>(a, nblocks, smem, st)
-                          : out_loss_launch<__nv_bfloat16, 3, true, true>(a, nblocks, smem, st);
-    return a.d_out == 1 ? out_loss_launch<float, 1, false, true>(a, nblocks, smem, st)
-                        : out_loss_launch<float, 3, false, true>(a, nblocks, smem, st);
+      return a.d_out == 1 ? out_loss_launch<__nv_bfloat16, 1, true, true>(h, a, nblocks, smem, st)
+                          : out_loss_launch<__nv_bfloat16, 3, true, true>(h, a, nblocks, smem, st);
+    return a.d_out == 1 ? out_loss_launch<float, 1, false, true>(h, a, nblocks, smem, st)
+                        : out_loss_launch<float, 3, false, true>(h, a, nblocks, smem, st);
   }
   if (prec == PINN_BF16)
-    return a.d_out == 1 ? out_loss_launch<__nv_bfloat16, 1, true, false>(a, nblocks, smem, st)
-                        : out_loss_launch<__nv_bfloat16, 3, true, false>(a, nblocks, smem, st);
-  return a.d_out == 1 ? out_loss_launch<float, 1, false, false>(a, nblocks, smem, st)
-                      : out_loss_launch<float, 3, false, false>(a, nblocks, smem, st);
+    return a.d_out == 1 ? out_loss_launch<__nv_bfloat16, 1, true, false>(h, a, nblocks, smem, st)
+                        : out_loss_launch<__nv_bfloat16, 3, true, false>(h, a, nblocks, smem, st);
+  return a.d_out == 1 ? out_loss_launch<float, 1, false, false>(h, a, nblocks, smem, st)
+                      : out_loss_launch<float, 3, false, false>(h, a, nblocks, smem, st);
 }
 
 

@@ -474,90 +474,85 @@ __global__ void __launch_bounds__(512 / TJ, TJ == 8 ? 4 : 2) k_f32_dw(const floa
 }
 
 template <int TJ>
-void f32_dw_launch(const void* Aop, const void* Bop, int M, int N, int64_t NC, int nsplit, int64_t kchunk, float* part,
-                   cudaStream_t st) {
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(k_f32_dw<TJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)W_SMEM);
-  (void)attr;   // a failure shows as the launch's error
+cudaError_t f32_dw_launch(pinn_handle* h, const void* Aop, const void* Bop, int M, int N, int64_t NC, int nsplit,
+                          int64_t kchunk, float* part, cudaStream_t st) {
+  const cudaError_t err = allow_smem(h, reinterpret_cast<const void*>(k_f32_dw<TJ>), W_SMEM);
+  if (err != cudaSuccess) return err;
   dim3 grid((N + WT - 1) / WT, (M + WT - 1) / WT, nsplit);
   k_f32_dw<TJ><<<grid, 512 / TJ, W_SMEM, st>>>((const float*)Aop, (const float*)Bop, M, N, NC, kchunk, part);
+  return cudaGetLastError();
 }
 
 template <int FM, int EPI, bool SINE>
-void f32_gemm_launch(const float* At, const void* Bop, int M, int K, int64_t NP, const EpiArgs& e, cudaStream_t st) {
+cudaError_t f32_gemm_launch(pinn_handle* h, const float* At, const void* Bop, int M, int K, int64_t NP, const EpiArgs& e,
+                            cudaStream_t st) {
   auto kern = k_f32_gemm<FM, EPI, SINE>;
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f32_smem<FM>());
-  (void)attr;   // a failure shows as the launch's error
+  const cudaError_t err = allow_smem(h, reinterpret_cast<const void*>(kern), f32_smem<FM>());
+  if (err != cudaSuccess) return err;
   kern<<<dim3((unsigned)(NP / FPTS), (M + FM - 1) / FM), 2 * FM, f32_smem<FM>(), st>>>(At, (const float*)Bop, M, K, e);
+  return cudaGetLastError();
 }
 
 // 128-feature blocks read each jet column half as often as 64-feature ones; they are
 // taken once they fill two blocks on every SM, below that the smaller blocks spread
 // the work over more SMs.
 template <int EPI, bool SINE>
-void f32_gemm(const float* At, const void* Bop, int M, int K, int64_t NP, const EpiArgs& e, int sms, cudaStream_t st) {
-  if (M > 64 && (NP / FPTS) * ((M + 127) / 128) >= 2 * (int64_t)sms)
-    f32_gemm_launch<128, EPI, SINE>(At, Bop, M, K, NP, e, st);
-  else
-    f32_gemm_launch<64, EPI, SINE>(At, Bop, M, K, NP, e, st);
+cudaError_t f32_gemm(pinn_handle* h, const float* At, const void* Bop, int M, int K, int64_t NP, const EpiArgs& e,
+                     cudaStream_t st) {
+  if (M > 64 && (NP / FPTS) * ((M + 127) / 128) >= 2 * (int64_t)h->sm_count)
+    return f32_gemm_launch<128, EPI, SINE>(h, At, Bop, M, K, NP, e, st);
+  return f32_gemm_launch<64, EPI, SINE>(h, At, Bop, M, K, NP, e, st);
 }
 
 }  // namespace
 
-void launch_simt_gemm_fwd(const float* W, const float* WT, const void* Bop, int M, int K, int64_t NP, const EpiArgs& e,
-                          int prec, int sms, cudaStream_t st) {
-  if (prec != PINN_BF16) {
-    if (e.act) f32_gemm<0, true>(WT, Bop, M, K, NP, e, sms, st);
-    else f32_gemm<0, false>(WT, Bop, M, K, NP, e, sms, st);
-    return;
-  }
+cudaError_t launch_simt_gemm_fwd(pinn_handle* h, const float* W, const float* WT, const void* Bop, int M, int K,
+                                 int64_t NP, const EpiArgs& e, int prec, cudaStream_t st) {
+  if (prec != PINN_BF16)
+    return e.act ? f32_gemm<0, true>(h, WT, Bop, M, K, NP, e, st) : f32_gemm<0, false>(h, WT, Bop, M, K, NP, e, st);
   dim3 grid((unsigned)(NP / TILE_PTS), (M + BM - 1) / BM);
   const __nv_bfloat16* B = (const __nv_bfloat16*)Bop;
   const __nv_bfloat16* Blo = (const __nv_bfloat16*)e.alo_in;
   if (e.act) k_simt_gemm<0, true><<<grid, THREADS, 0, st>>>(W, B, Blo, M, K, NP, e);
   else k_simt_gemm<0, false><<<grid, THREADS, 0, st>>>(W, B, Blo, M, K, NP, e);
+  return cudaGetLastError();
 }
 
-void launch_simt_gemm_adj(const float* WT, const float* W, const void* Bop, int M, int K, int64_t NP, const EpiArgs& e,
-                          int prec, int sms, cudaStream_t st) {
-  if (prec != PINN_BF16) {
-    if (e.act) f32_gemm<1, true>(W, Bop, M, K, NP, e, sms, st);
-    else f32_gemm<1, false>(W, Bop, M, K, NP, e, sms, st);
-    return;
-  }
+cudaError_t launch_simt_gemm_adj(pinn_handle* h, const float* WT, const float* W, const void* Bop, int M, int K,
+                                 int64_t NP, const EpiArgs& e, int prec, cudaStream_t st) {
+  if (prec != PINN_BF16)
+    return e.act ? f32_gemm<1, true>(h, W, Bop, M, K, NP, e, st) : f32_gemm<1, false>(h, W, Bop, M, K, NP, e, st);
   dim3 grid((unsigned)(NP / TILE_PTS), (M + BM - 1) / BM);
   const __nv_bfloat16* B = (const __nv_bfloat16*)Bop;
   if (e.act) k_simt_gemm<1, true><<<grid, THREADS, 0, st>>>(WT, B, nullptr, M, K, NP, e);
   else k_simt_gemm<1, false><<<grid, THREADS, 0, st>>>(WT, B, nullptr, M, K, NP, e);
+  return cudaGetLastError();
 }
 
-void launch_simt_gemm_lin(const float* WT, const float* W, const void* Bop, int M, int K, int64_t NP, void* out,
-                          int prec, int sms, cudaStream_t st) {
+cudaError_t launch_simt_gemm_lin(pinn_handle* h, const float* WT, const float* W, const void* Bop, int M, int K,
+                                 int64_t NP, void* out, int prec, cudaStream_t st) {
   EpiArgs e{};
   e.out = out;
-  if (prec != PINN_BF16) {
-    f32_gemm<2, false>(W, Bop, M, K, NP, e, sms, st);
-    return;
-  }
+  if (prec != PINN_BF16) return f32_gemm<2, false>(h, W, Bop, M, K, NP, e, st);
   dim3 grid((unsigned)(NP / TILE_PTS), (M + BM - 1) / BM);
   k_simt_gemm<2, false><<<grid, THREADS, 0, st>>>(WT, (const __nv_bfloat16*)Bop, nullptr, M, K, NP, e);
+  return cudaGetLastError();
 }
 
-void launch_simt_gemm_dw(const void* Aop, const void* Bop, int M, int N, int64_t NC, int nsplit, float* part, int prec,
-                         cudaStream_t st) {
+cudaError_t launch_simt_gemm_dw(pinn_handle* h, const void* Aop, const void* Bop, int M, int N, int64_t NC, int nsplit,
+                                float* part, int prec, cudaStream_t st) {
   const int64_t per = (NC + nsplit - 1) / nsplit;
   const int64_t kchunk = (per + DBK - 1) / DBK * DBK;
   if (prec != PINN_BF16) {
     // Short splits (a few stages per block, few blocks) are bound by latency: twice the
     // threads per block, half the columns each (4x64 network at 4,608 points: 13 us per launch
     // against 17; at 17,408 points and 256 wide 0.28 ms against 0.24).
-    if (kchunk <= 8 * DBK) f32_dw_launch<4>(Aop, Bop, M, N, NC, nsplit, kchunk, part, st);
-    else f32_dw_launch<8>(Aop, Bop, M, N, NC, nsplit, kchunk, part, st);
-    return;
+    return kchunk <= 8 * DBK ? f32_dw_launch<4>(h, Aop, Bop, M, N, NC, nsplit, kchunk, part, st)
+                             : f32_dw_launch<8>(h, Aop, Bop, M, N, NC, nsplit, kchunk, part, st);
   }
   dim3 grid((N + DBN - 1) / DBN, (M + DBM - 1) / DBM, nsplit);
   k_simt_dw<<<grid, THREADS, 0, st>>>((const __nv_bfloat16*)Aop, (const __nv_bfloat16*)Bop, M, N, NC, kchunk, part);
+  return cudaGetLastError();
 }
 
 }  // namespace pinn

@@ -1006,17 +1006,11 @@ bool tc_map3(CUtensorMap* m, const void* base, bool fp32, uint64_t tcols, uint64
 
 namespace {
 
-// Reserves the dynamic shared memory of kernel `kern` once per kernel.
 template <typename K>
-pinn_status reserve_smem(pinn_handle* h, K kern, size_t bytes, bool& done, const char* what) {
-  if (done) return PINN_OK;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) {
-    cudaGetLastError();   // do not leave the failure for the next launch to report
-    snprintf(h->err, sizeof(h->err), "%s: cannot reserve %zu bytes of shared memory", what, bytes);
-    return PINN_ERR_CUDA;
-  }
-  done = true;
-  return PINN_OK;
+pinn_status reserve_smem(pinn_handle* h, K kern, size_t bytes, const char* what) {
+  if (allow_smem(h, reinterpret_cast<const void*>(kern), bytes) == cudaSuccess) return PINN_OK;
+  snprintf(h->err, sizeof(h->err), "%s: cannot reserve %zu bytes of shared memory", what, bytes);
+  return PINN_ERR_CUDA;
 }
 
 pinn_status launch_check(pinn_handle* h, const char* what) {
@@ -1031,8 +1025,7 @@ template <bool TF32, int MODE, bool SPLIT, bool SINE>
 pinn_status launch_group(pinn_handle* h, const TcGroupEntry* d_tab, int n, int blocks, cudaStream_t st) {
   using C = Cfg<TF32, MODE, SPLIT>;
   auto kern = k_tc_gemm_group<TF32, MODE, SPLIT, SINE>;
-  static bool attr_set = false;   // per instantiation
-  pinn_status s = reserve_smem(h, kern, C::SMEM, attr_set, "grouped tcgen05 kernel");
+  pinn_status s = reserve_smem(h, kern, C::SMEM, "grouped tcgen05 kernel");
   if (s) return s;
   kern<<<blocks, C::NTHREADS, C::SMEM, st>>>(d_tab, n);
   return launch_check(h, "grouped tcgen05 kernel");
@@ -1079,8 +1072,7 @@ pinn_status launch(pinn_handle* h, const CUtensorMap& a, const CUtensorMap& a2, 
   }
   using C = Cfg<TF32, MODE, SPLIT>;
   auto kern = k_tc_gemm<TF32, MODE, SPLIT, SINE>;
-  static bool attr_set = false;   // per instantiation
-  pinn_status s = reserve_smem(h, kern, C::SMEM, attr_set, "tcgen05 kernel");
+  pinn_status s = reserve_smem(h, kern, C::SMEM, "tcgen05 kernel");
   if (s) return s;
   kern<<<grid, C::NTHREADS, C::SMEM, st>>>(a, a2, b, blo, p);
   return launch_check(h, "tcgen05 kernel");
@@ -1192,8 +1184,7 @@ pinn_status fwd_impl(pinn_handle* h, const void* W, const void* Wlo, const void*
       if (!make_map3(&mo, e.out, false, TILE_COLS, fout, nt, TILE_PTS, BM) ||
           (e.alo_out && !make_map3(&mol, e.alo_out, false, TILE_PTS, fout, nt, TILE_PTS, BM)))
         return map_err(h, "paired forward outputs");
-      static bool attr_set = false;
-      pinn_status s = reserve_smem(h, k_tc_fwd_pair, P::SMEM, attr_set, "paired forward kernel");
+      pinn_status s = reserve_smem(h, k_tc_fwd_pair, P::SMEM, "paired forward kernel");
       if (s) return s;
       k_tc_fwd_pair<<<grid & ~1, P::NTHREADS, P::SMEM, st>>>(ma, ma2, mb, mlo, mv, mo, mol, p);
       return launch_check(h, "paired forward");
@@ -1680,8 +1671,7 @@ namespace {
 
 template <bool DW>
 pinn_status launch_adjdw_group(pinn_handle* h, const TcGroupEntry* d_tab, int n, int blocks, cudaStream_t st) {
-  static bool attr_set = false;   // per instantiation
-  pinn_status s = reserve_smem(h, k_tc_adjdw_group<DW>, FzCfg<DW>::SMEM, attr_set, "grouped fused adjoint kernel");
+  pinn_status s = reserve_smem(h, k_tc_adjdw_group<DW>, FzCfg<DW>::SMEM, "grouped fused adjoint kernel");
   if (s) return s;
   k_tc_adjdw_group<DW><<<blocks, FZ_NT, FzCfg<DW>::SMEM, st>>>(d_tab, n);
   return launch_check(h, "grouped fused adjoint");
@@ -1694,8 +1684,7 @@ pinn_status launch_adjdw(pinn_handle* h, const CUtensorMap& w, const CUtensorMap
     const CUtensorMap maps[4] = {w, z, a, o};
     return batch_add(h->tc_batch, &launch_adjdw_group<DW>, maps, 4, p, grid);
   }
-  static bool attr_set = false;   // per instantiation
-  pinn_status s = reserve_smem(h, k_tc_adjdw<DW>, FzCfg<DW>::SMEM, attr_set, "fused adjoint kernel");
+  pinn_status s = reserve_smem(h, k_tc_adjdw<DW>, FzCfg<DW>::SMEM, "fused adjoint kernel");
   if (s) return s;
   k_tc_adjdw<DW><<<grid, FZ_NT, FzCfg<DW>::SMEM, st>>>(w, z, a, o, p);
   return launch_check(h, "fused adjoint");
@@ -2167,9 +2156,8 @@ pinn_status tc_gemm_fwd_all(pinn_handle* h, const TcFwdLayer* layers, int n, con
   p.wlo_values_only = (h->spec.flags & PINN_FLAG_BF16_VALUE_SPLIT) ? 1 : 0;
   p.status = h->d_status;
   p.wait_ns = WAIT_NS;
-  static bool attr_set[2] = {false, false};
   auto kern = m2 ? k_tc_fwd_all<true> : k_tc_fwd_all<false>;
-  const pinn_status s = reserve_smem(h, kern, FF_SMEM, attr_set[m2 ? 1 : 0], "fused forward kernel");
+  const pinn_status s = reserve_smem(h, kern, FF_SMEM, "fused forward kernel");
   if (s) return s;
   kern<<<grid_for(h, p.ntiles), FF_NT, FF_SMEM, st>>>(p);
   return launch_check(h, "fused forward");
