@@ -429,47 +429,53 @@ template <> __device__ __forceinline__ void store4_stream<__nv_bfloat16>(__nv_bf
   __stcs(reinterpret_cast<uint2*>(p), u);
 }
 
-// Temporal causality, first pass: the segment sums of squared residuals.  Each warp keeps
-// its own sums in shared memory, SEG_WORDS floats: lane s owns segment s (at most 32) and
-// adds the warp's 16 points of a tile in order, as compensated FP32 pairs (exact to about
-// 2^-48, like the FP64 sums they become at the end of the block).  The points' squared
-// residuals and segment come from the 16 float4 staged after the sums.  (One thread adding all
-// 64 points of a tile in FP64, with the block waiting at two barriers, was most of the pass:
-// both output passes of a 4x128 network at 17,408 points 0.156 -> 0.062 ms.)
-constexpr int SEG_SUMS = 7 * CAUSAL_MAX;            // 3 equations x (sum, compensation), count
+// Temporal causality, first pass: the segment sums of squared residuals, in FP64 (a segment's
+// sum may pass the FP32 range that its terms are in).  Each warp keeps its own sums in shared
+// memory, SEG_WORDS 32-bit words: lane s owns segment s (at most 32) and adds those of the
+// warp's 16 points of a tile that are its own, in order.  FP64 is a slow pipe on this part, so
+// a lane visits only its own points: the warp issues as many additions as its fullest segment
+// has points, not 16.  The points' squared residuals and segment come from the 16 float4 staged
+// after the sums.  (One thread adding all 64 points of a tile in FP64, with the block waiting at
+// two barriers, was most of the pass: both output passes of a 4x128 network at 17,408 points
+// 0.156 -> 0.062 ms; compensated FP32 pairs took as long as this, 157 us for the whole step.)
+constexpr int SEG_SUMS = 7 * CAUSAL_MAX;            // 3 equations (FP64), count
 constexpr int SEG_WORDS = SEG_SUMS + 4 * 16;
 
+__device__ __forceinline__ double* seg_sum(float* sw, int k) { return reinterpret_cast<double*>(sw) + k * CAUSAL_MAX; }
+__device__ __forceinline__ unsigned* seg_count(float* sw) { return reinterpret_cast<unsigned*>(sw + 6 * CAUSAL_MAX); }
 __device__ __forceinline__ float4* seg_points(float* sw) { return reinterpret_cast<float4*>(sw + SEG_SUMS); }
 __device__ __forceinline__ void seg_clear(float* sw, int lane) {
 #pragma unroll
-  for (int k = 0; k < 7; ++k) sw[k * CAUSAL_MAX + lane] = 0.f;
+  for (int k = 0; k < 3; ++k) seg_sum(sw, k)[lane] = 0.0;
+  seg_count(sw)[lane] = 0u;
 }
 __device__ __forceinline__ void seg_add(float* sw, int lane) {
   __syncwarp();
-  Acc2 a[3];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) { a[k].s = sw[(2 * k) * CAUSAL_MAX + lane]; a[k].c = sw[(2 * k + 1) * CAUSAL_MAX + lane]; }
-  float n = sw[6 * CAUSAL_MAX + lane];
   const float4* pts = seg_points(sw);
-#pragma unroll 4
-  for (int q = 0; q < 16; ++q) {
-    const float4 v = pts[q];
-    const bool mine = __float_as_int(v.w) == lane;
-    a[0].add(mine ? v.x : 0.f); a[1].add(mine ? v.y : 0.f); a[2].add(mine ? v.z : 0.f);
-    n += mine ? 1.f : 0.f;
-  }
+  unsigned mine = 0u;
 #pragma unroll
-  for (int k = 0; k < 3; ++k) { sw[(2 * k) * CAUSAL_MAX + lane] = a[k].s; sw[(2 * k + 1) * CAUSAL_MAX + lane] = a[k].c; }
-  sw[6 * CAUSAL_MAX + lane] = n;
+  for (int q = 0; q < 16; ++q) mine |= (unsigned)(__float_as_int(pts[q].w) == lane) << q;
+  if (mine) {
+    double s[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) s[k] = seg_sum(sw, k)[lane];
+    seg_count(sw)[lane] += __popc(mine);
+    do {
+      const float4 v = pts[__ffs(mine) - 1];
+      s[0] += v.x; s[1] += v.y; s[2] += v.z;
+      mine &= mine - 1u;
+    } while (mine);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) seg_sum(sw, k)[lane] = s[k];
+  }
   __syncwarp();
 }
 // The block's sums of segment s, column k (3 equations, count): four warps in order.
-__device__ __forceinline__ double seg_total(const float* sw0, int stride, int s, int k) {
+__device__ __forceinline__ double seg_total(float* sw0, int stride, int s, int k) {
   double t = 0.0;
   for (int w = 0; w < 4; ++w) {
-    const float* sw = sw0 + w * stride;
-    t += k == 3 ? (double)sw[6 * CAUSAL_MAX + s]
-                : (double)sw[(2 * k) * CAUSAL_MAX + s] + (double)sw[(2 * k + 1) * CAUSAL_MAX + s];
+    float* sw = sw0 + w * stride;
+    t += k == 3 ? (double)seg_count(sw)[s] : seg_sum(sw, k)[s];
   }
   return t;
 }
@@ -1554,7 +1560,7 @@ __global__ void __launch_bounds__(OT_THREADS, 2) k_out_loss_mma(const __grid_con
     cons_sync();
     for (int i = threadIdx.x; i < CAUSAL_MAX * 4; i += OT_CONS)
       a.segpart[(int64_t)blockIdx.x * CAUSAL_MAX * 4 + i] =
-          seg_total(reinterpret_cast<const float*>(ring + lay.stg + 768), OM_SCRATCH / 4, i / 4, i % 4);
+          seg_total(reinterpret_cast<float*>(ring + lay.stg + 768), OM_SCRATCH / 4, i / 4, i % 4);
   }
   if (!a.want_grad) return;
   cons_sync();

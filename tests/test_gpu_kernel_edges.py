@@ -171,3 +171,37 @@ def test_tf32_edges(cuda_lib, pde, widths, ff, n_res):
     rt, rg = run_oracle(spec, p, B, b, prob, chunk=4096)
     assert abs(gt[0] - rt[0]) <= TOL["tf32"] * abs(rt[0])
     assert np.linalg.norm(gg - rg) <= 2.0 ** -9 * np.linalg.norm(rg)
+
+
+@pytest.mark.parametrize("widths,precision", [([13, 13], "fp32"), ([64, 64], "bf16"), ([8, 288], "bf16")])
+def test_causal_segment_sums_beyond_fp32(cuda_lib, widths, precision):
+    """A segment whose squared residuals are FP32 numbers but whose sum is not, in each of the
+    three output kernels: the loss stays finite, the later segment's weight is 0 and no NaN."""
+    import oracle
+    from paper_2604_15645_gb300 import api
+    from parity_blocks import param_blocks
+    spec = NetSpec(PDE_BURGERS, 2, 1, widths)
+    p = init_params(spec, 81, 0.2)
+    b = make_batch(PDE_BURGERS, 2000, 40, 30, 82, 83)
+    cz = dict(segments=2, eps=1.5, t_index=1, t0=0.0, t1=1.0)
+    last = slice(*{n: (s, e) for n, s, e in param_blocks(spec)}["V3"][:2])
+
+    def ref(scale):
+        q = np.array(p, dtype=np.float32)
+        q[last] *= scale
+        return q, *oracle.loss_and_grad(oracle.Model.from_spec(spec), q, None, b, 0.05, (0.01, 0.0, 0.0), causal=cz)
+
+    # u u_x is all of the residual: scale the output layer to a mean square of 4e37 in the
+    # first segment (the sums of its points among a warp's 16 reach 5e38 to 7e38, no point 1.2e38)
+    _, t, _ = ref(1e9)
+    q, terms, rg = ref(np.float32(1e9 * (2e37 / t["pde"]) ** 0.25))   # pde = half of that mean
+    assert list(terms["causal_weights"]) == [1.0, 0.0]
+    net = api.PinnNet.from_spec(spec, precision)
+    net.set_causal(2, 1.5)
+    out, g = net.loss_grad(torch.tensor(q, device="cuda"), api.DeviceBatch.from_host(b), api.make_problem(0.05, 0.01, 0.0, 0.0))
+    torch.cuda.synchronize()
+    assert net.status_poll() == 0
+    tol = TOL[precision]
+    assert abs(float(out[0]) - terms["total"]) <= tol * terms["total"]
+    assert net.causal_weights().cpu().tolist() == [1.0, 0.0]
+    assert np.linalg.norm(g.cpu().numpy().astype(np.float64) - rg) <= tol * np.linalg.norm(rg)
