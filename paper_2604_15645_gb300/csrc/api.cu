@@ -7,6 +7,9 @@
 #include <cstring>
 #include <new>
 
+#include <cuda.h>
+#include <cudaTypedefs.h>
+
 #include "internal.h"
 #include "tc.h"
 
@@ -59,8 +62,25 @@ int pde_dout(int pde) { return (pde == PINN_NS_STEADY_2D || pde == PINN_MAXWELL_
 
 namespace pinn {
 
+void share_smem_limits(pinn_handle* h) {
+  static ContextLimits limits;
+  auto entry = [](const char* name, unsigned version) -> void* {
+    cudaDriverEntryPointQueryResult q;
+    void* fn = nullptr;
+    const cudaError_t e = cudaGetDriverEntryPointByVersion(name, &fn, version, cudaEnableDefault, &q);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess && q == cudaDriverEntryPointSuccess ? fn : nullptr;
+  };
+  static const auto get_current = reinterpret_cast<PFN_cuCtxGetCurrent_v4000>(entry("cuCtxGetCurrent", 4000));
+  static const auto get_id = reinterpret_cast<PFN_cuCtxGetId_v12000>(entry("cuCtxGetId", 12000));
+  CUcontext ctx = nullptr;
+  unsigned long long id = 0;
+  if (!get_current || !get_id || get_current(&ctx) != CUDA_SUCCESS || !ctx || get_id(ctx, &id) != CUDA_SUCCESS) return;
+  if (SmemLimits* shared = limits.of(id)) h->smem = shared;
+}
+
 cudaError_t allow_smem(pinn_handle* h, const void* kern, size_t bytes) {
-  return h->smem.allow(kern, bytes, cudaSuccess, cudaErrorInvalidValue, [&](size_t* limit) {
+  return h->smem->allow(kern, bytes, cudaSuccess, cudaErrorInvalidValue, [&](size_t* limit) {
     cudaFuncAttributes fa;
     int optin = 0;
     cudaError_t e = cudaFuncGetAttributes(&fa, kern);
@@ -913,6 +933,7 @@ pinn_status pinn_create(const pinn_spec* spec, pinn_handle** out) {
     delete h;
     return e == cudaErrorMemoryAllocation ? PINN_ERR_OOM : PINN_ERR_CUDA;
   }
+  share_smem_limits(h);
   tc_init(h);
   *out = h;
   return PINN_OK;

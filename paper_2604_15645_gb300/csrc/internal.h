@@ -81,7 +81,9 @@ struct pinn_graph_key {
 
 struct pinn_handle {
   pinn_spec spec{};
-  pinn::SmemLimits smem;     // kernels whose shared-memory limit has been raised for this handle
+  // kernels whose shared-memory limit has been raised: the context's record (else the handle's own)
+  pinn::SmemLimits own_smem;
+  pinn::SmemLimits* smem = &own_smem;
   int d_in = 0, d_out = 0, L = 0;
   int jet_mode = 0;
   int first_gemm = 0;        // index of the first hidden layer computed by a GEMM (0 with FF, 1 without)
@@ -123,6 +125,8 @@ namespace pinn {
 
 // Before a launch of `kern` with `bytes` of dynamic shared memory (see smem_limit.h).
 cudaError_t allow_smem(pinn_handle* h, const void* kern, size_t bytes);
+// Attaches a new handle to the current context's record.
+void share_smem_limits(pinn_handle* h);
 
 pinn_status make_plan(const pinn_handle* h, int64_t n_res, int64_t n_ic, int64_t n_bc, Plan* plan);
 

@@ -83,3 +83,56 @@ def test_no_limit_is_kept_per_process():
     found = {f: open(os.path.join(csrc, f)).read().count("cudaFuncSetAttribute(")
              for f in sorted(os.listdir(csrc)) if f.endswith((".cu", ".cuh", ".h"))}
     assert {f: n for f, n in found.items() if n} == {"api.cu": 1}
+
+
+SHARED = r"""
+#include <cstdio>
+#include <thread>
+#include <vector>
+#include "smem_limit.h"
+#define CHECK(x) do { if (!(x)) { printf("failed: %s\n", #x); return 1; } } while (0)
+
+int main() {
+  static pinn::ContextLimits contexts;
+  static int kern[96];
+  pinn::SmemLimits* a = contexts.of(7);
+  CHECK(a && contexts.of(8) && contexts.of(8) != a && contexts.of(7) == a);   // one record per context
+  std::atomic<int> raised{0}, wrong{0};
+  std::vector<std::thread> threads;
+  for (int t = 0; t < 8; ++t)
+    threads.emplace_back([&] {
+      pinn::SmemLimits* mine = contexts.of(7);
+      for (int r = 0; r < 200; ++r)
+        for (int i = 0; i < 96; ++i)
+          wrong += mine->allow(&kern[i], (size_t)(1000 + i), 0, 9, [&](size_t* limit) {
+            ++raised;
+            *limit = (size_t)(1000 + i);
+            return 0;
+          }) != 0;
+    });
+  for (auto& t : threads) t.join();
+  CHECK(wrong == 0 && raised >= 96 && raised <= 8 * 96);
+  const int before = raised;
+  for (int i = 0; i < 96; ++i)   // what one handle raised serves the context's next one
+    CHECK(contexts.of(7)->allow(&kern[i], 1000, 0, 9, [&](size_t*) { ++raised; return 2; }) == 0);
+  CHECK(raised == before);
+  CHECK(contexts.of(8)->allow(&kern[0], 1000, 0, 9, [&](size_t*) { return 2; }) == 2);   // not another context's
+  int more = 0;
+  for (uint64_t c = 100; c < 200; ++c) more += contexts.of(c) != nullptr;
+  CHECK(more == 30 && contexts.of(7) == a);   // bounded; the known ones stay
+  printf("ok\n");
+  return 0;
+}
+"""
+
+
+def test_handles_of_a_context_share_its_record(tmp_path):
+    cxx = shutil.which("g++")
+    if not cxx:
+        pytest.skip("no C++ compiler")
+    src, exe = tmp_path / "shared.cpp", tmp_path / "shared"
+    src.write_text(SHARED)
+    subprocess.run([cxx, "-std=c++17", "-O1", "-pthread", "-Wall", "-Werror", "-I",
+                    os.path.join(ROOT, "paper_2604_15645_gb300", "csrc"), str(src), "-o", str(exe)], check=True, timeout=300)
+    r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=60)
+    assert r.returncode == 0 and r.stdout.strip() == "ok", r.stdout
