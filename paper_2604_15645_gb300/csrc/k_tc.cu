@@ -40,6 +40,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "fwd_route.h"
 #include "jet.cuh"
 #include "ptx.cuh"
 #include "tc.h"
@@ -1078,9 +1079,10 @@ pinn_status launch(pinn_handle* h, const CUtensorMap& a, const CUtensorMap& a2, 
   return launch_check(h, "tcgen05 kernel");
 }
 
-// Whether a launch runs in pairs: two m-tiles of a column tile side by side, so an even
-// number of them (and not in a grouped launch, whose entries start at any block).
-bool in_pairs(const pinn_handle* h, const TcParams& p) { return !h->tc_batch && p.m_tiles % 2 == 0 && h->sm_count >= 2; }
+// Whether a launch runs in pairs (not in a grouped launch, whose entries start at any block).
+bool in_pairs(const pinn_handle* h, const TcParams& p) {
+  return !h->tc_batch && fwd_in_pairs(p.m_tiles, p.n_tiles, p.K, p.wlo_values_only != 0, h->sm_count);
+}
 
 int grid_for(const pinn_handle* h, int tiles) { return std::max(1, std::min(tiles, std::max(h->sm_count, 1))); }
 

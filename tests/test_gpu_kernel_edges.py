@@ -205,3 +205,30 @@ def test_causal_segment_sums_beyond_fp32(cuda_lib, widths, precision):
     assert abs(float(out[0]) - terms["total"]) <= tol * terms["total"]
     assert net.causal_weights().cpu().tolist() == [1.0, 0.0]
     assert np.linalg.norm(g.cpu().numpy().astype(np.float64) - rg) <= tol * np.linalg.norm(rg)
+
+
+@pytest.mark.parametrize("widths,value_split", [
+    ([512, 1000, 256], False),        # eight m-tiles, the last of 104 rows; two on a K of 15.6 chunks
+    ([384, 512, 200], True),          # four m-tiles; two, the second of 72 rows
+])
+def test_paired_forward_sizes(cuda_lib, monkeypatch, widths, value_split):
+    """The forward in pairs of CTAs, at sizes that its dispatch gives it, bitwise against the
+    unpaired launches (which the grouped many-network step runs)."""
+    from paper_2604_15645_gb300 import _lib, api
+    spec = NetSpec(PDE_MAXWELL, 3, 3, widths, rwf=True)
+    p, n_res = init_params(spec, 91, 0.2), 30100
+    db = api.DeviceBatch.from_host(make_batch(PDE_MAXWELL, n_res, 30, 20, 93, 94))
+    prob = api.make_problem(0.02)
+    net = api.PinnNet.from_spec(spec, "bf16", value_split=value_split)
+    loss, grad = net.loss_grad(torch.tensor(p, device="cuda"), db, prob)
+    make_spec, flags = _lib.make_spec, _lib.PINN_FLAG_BF16_VALUE_SPLIT if value_split else 0
+    monkeypatch.setattr(_lib, "make_spec", lambda *args: make_spec(*args, flags))
+    multi = api.PinnMulti([spec], "bf16")
+    multi.set_inputs([db], [prob])
+    multi.grouped = True
+    q = torch.tensor(p, device="cuda")
+    g, m, v = (torch.zeros_like(q) for _ in range(3))
+    ref = multi.train_step(q, g, m, v, step=1)
+    torch.cuda.synchronize()
+    assert net.status_poll() == 0 and multi.status_poll() == 0
+    assert torch.equal(loss, ref[0]) and torch.equal(grad, g)
