@@ -23,4 +23,11 @@ inline bool fwd_in_pairs(int m_tiles, int n_tiles, int K, bool wlo_values_only, 
          (int64_t)m_tiles * n_tiles >= 6 * (int64_t)sm_count;
 }
 
+// Whether a network's hidden GEMM layers (all at most 256 wide) run in one kernel
+// (k_tc_fwd_all).  With a single layer there is nothing to keep in shared memory, and the layer's
+// two m-tiles follow each other in one CTA: the layer's own launch is faster at every size
+// (256 wide, K = 128, 3,000 points: 35.5 against 40.2 us for the loss; 40,000: 79.0 against 90.5;
+// 128 wide 31.4 against 33.2 and 58.3 against 60.3).
+inline bool fwd_in_one_kernel(int layers) { return layers >= 2; }
+
 }  // namespace pinn

@@ -2130,7 +2130,7 @@ __global__ void __launch_bounds__(FF_NT, 1) k_tc_fwd_all(const __grid_constant__
 }  // namespace
 
 bool tc_fwd_all_supported(const pinn_handle* h, int64_t NC) {
-  if (h->spec.precision != PINN_BF16 || h->act != PINN_ACT_TANH || h->first_gemm >= h->L) return false;
+  if (h->spec.precision != PINN_BF16 || h->act != PINN_ACT_TANH || !fwd_in_one_kernel(h->L - h->first_gemm)) return false;
   for (int li = h->first_gemm; li < h->L; ++li)
     if (!tc_layer_supported(h, li, NC) || h->layers[li].fin > 256 || h->layers[li].fout > 256) return false;
   return true;

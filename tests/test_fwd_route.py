@@ -35,3 +35,7 @@ def test_pairs_only_where_they_are_faster(tmp_path):
     exprs = [f"fwd_in_pairs({(w + 127) // 128}, {(n + 63) // 64}, {k}, {str(v).lower()}, 152)" for w, k, n, v, _ in cases]
     exprs += ["fwd_in_pairs(4, 1 << 30, 512, false, 152)", "fwd_in_pairs(4, 100000, 512, false, 1)"]
     assert _eval(tmp_path, exprs) == [c[4] for c in cases] + [True, False]
+
+
+def test_one_kernel_needs_more_than_one_layer(tmp_path):
+    assert _eval(tmp_path, [f"fwd_in_one_kernel({n})" for n in (0, 1, 2, 3, 16)]) == [False, False, True, True, True]

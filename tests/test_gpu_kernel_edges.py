@@ -232,3 +232,32 @@ def test_paired_forward_sizes(cuda_lib, monkeypatch, widths, value_split):
     torch.cuda.synchronize()
     assert net.status_poll() == 0 and multi.status_poll() == 0
     assert torch.equal(loss, ref[0]) and torch.equal(grad, g)
+
+
+@pytest.mark.parametrize("widths,ff", [([136, 256], 0), ([200], 64), ([64, 16], 0)])
+@pytest.mark.parametrize("n_res", [1, 20000])
+def test_single_gemm_layer(cuda_lib, widths, ff, n_res):
+    """One hidden GEMM layer runs its own forward launch: bitwise the grouped launch's loss and
+    gradient, and the same loss without a gradient."""
+    from paper_2604_15645_gb300 import api
+    spec = NetSpec(PDE_BURGERS, 2, 1, widths, ff_m=ff, ff_sigma=1.0, rwf=True)
+    p, B = init_params(spec, 91, 0.2), ff_matrix(spec, 92)
+    prob, db = api.make_problem(0.02), api.DeviceBatch.from_host(make_batch(PDE_BURGERS, n_res, 30, 20, 93, 94))
+    Bd = None if B is None else torch.tensor(B, device="cuda")
+    multi = api.PinnMulti([spec], "bf16")
+    net = api.PinnNet.from_spec(spec, "bf16")
+    if Bd is not None:
+        api._lib.check_multi(api._lib.load().pinn_multi_set_ff_matrix(multi.h, 0, Bd.data_ptr()), multi.h)
+        net.set_ff_matrix(B)
+    multi.set_inputs([db], [prob])
+    multi.grouped = True
+    q = torch.tensor(p, device="cuda")
+    g, m, v = (torch.zeros_like(q) for _ in range(3))
+    ref = multi.train_step(q, g, m, v, step=1)
+    params = torch.tensor(p, device="cuda")
+    terms, grad = net.loss_grad(params, db, prob)
+    terms = terms.clone()
+    loss = net.loss(params, db, prob)
+    torch.cuda.synchronize()
+    assert net.status_poll() == 0 and multi.status_poll() == 0
+    assert torch.equal(terms, ref[0]) and torch.equal(grad, g) and torch.equal(loss, terms)
