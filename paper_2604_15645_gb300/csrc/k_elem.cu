@@ -431,13 +431,13 @@ template <> __device__ __forceinline__ void store4_stream<__nv_bfloat16>(__nv_bf
 
 // Temporal causality, first pass: the segment sums of squared residuals, in FP64 (a segment's
 // sum may pass the FP32 range that its terms are in).  Each warp keeps its own sums in shared
-// memory, SEG_WORDS 32-bit words: lane s owns segment s (at most 32) and adds those of the
-// warp's 16 points of a tile that are its own, in order.  FP64 is a slow pipe on this part, so
-// a lane visits only its own points: the warp issues as many additions as its fullest segment
-// has points, not 16.  The points' squared residuals and segment come from the 16 float4 staged
-// after the sums.  (One thread adding all 64 points of a tile in FP64, with the block waiting at
-// two barriers, was most of the pass: both output passes of a 4x128 network at 17,408 points
-// 0.156 -> 0.062 ms; compensated FP32 pairs took as long as this, 157 us for the whole step.)
+// memory, SEG_WORDS 32-bit words, for at most 32 segments.  The warp's 16 points of a tile, staged
+// after the sums, are added up per segment first: lane q holds point q and the next lane of
+// its segment, and doubling steps leave a segment's sum in its first lane (a fixed order).  FP64 is a
+// slow pipe on this part: at most 5 additions per equation instead of one per point.
+// (One thread adding all 64 points of a tile in FP64, with the block waiting at two barriers,
+// was most of the pass: both output passes of a 4x128 network at 17,408 points 0.156 ->
+// 0.062 ms; compensated FP32 pairs took as long as this, 157 us for the whole step.)
 constexpr int SEG_SUMS = 7 * CAUSAL_MAX;            // 3 equations (FP64), count
 constexpr int SEG_WORDS = SEG_SUMS + 4 * 16;
 
@@ -449,24 +449,30 @@ __device__ __forceinline__ void seg_clear(float* sw, int lane) {
   for (int k = 0; k < 3; ++k) seg_sum(sw, k)[lane] = 0.0;
   seg_count(sw)[lane] = 0u;
 }
+template <int D>
 __device__ __forceinline__ void seg_add(float* sw, int lane) {
+  constexpr int EQS = D == 1 ? 1 : 3;
   __syncwarp();
-  const float4* pts = seg_points(sw);
-  unsigned mine = 0u;
+  const float4 v = seg_points(sw)[lane & 15];
+  const int seg = lane < 16 ? __float_as_int(v.w) : -1;   // (-1: not an interior point)
+  const unsigned peers = __match_any_sync(0xffffffffu, seg);
+  const unsigned after = peers & (0xfffffffeu << lane);
+  int next = seg >= 0 && after ? __ffs(after) - 1 : -1;
+  double s[3] = {v.x, v.y, v.z};
+  // s is the sum of the segment's lanes from this one up to before `next`
+  while (__any_sync(0xffffffffu, next >= 0)) {
+    const int from = next >= 0 ? next : lane;
 #pragma unroll
-  for (int q = 0; q < 16; ++q) mine |= (unsigned)(__float_as_int(pts[q].w) == lane) << q;
-  if (mine) {
-    double s[3];
+    for (int k = 0; k < EQS; ++k) {
+      const double t = __shfl_sync(0xffffffffu, s[k], from);
+      if (next >= 0) s[k] += t;
+    }
+    next = __shfl_sync(0xffffffffu, next, from);
+  }
+  if (seg >= 0 && lane == __ffs(peers) - 1) {
 #pragma unroll
-    for (int k = 0; k < 3; ++k) s[k] = seg_sum(sw, k)[lane];
-    seg_count(sw)[lane] += __popc(mine);
-    do {
-      const float4 v = pts[__ffs(mine) - 1];
-      s[0] += v.x; s[1] += v.y; s[2] += v.z;
-      mine &= mine - 1u;
-    } while (mine);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) seg_sum(sw, k)[lane] = s[k];
+    for (int k = 0; k < EQS; ++k) seg_sum(sw, k)[seg] += s[k];
+    seg_count(sw)[seg] += __popc(peers);
   }
   __syncwarp();
 }
@@ -578,7 +584,7 @@ __global__ void __launch_bounds__(OUT_THREADS) k_out_loss(OutArgs a) {
 #pragma unroll
         for (int j = 0; j < 4; ++j)
           seg_points(s_seg[warp])[(q0 & 15) + j] = make_float4(rrj[j][0], rrj[j][1], rrj[j][2], __int_as_float(segj[j]));
-      seg_add(s_seg[warp], lane);
+      seg_add<D>(s_seg[warp], lane);
     }
     if (!a.want_grad) continue;
     if (sl == 0) {
@@ -926,7 +932,7 @@ __global__ void __launch_bounds__(OT_THREADS) k_out_loss_tma(const __grid_consta
 #pragma unroll
         for (int j = 0; j < 4; ++j)
           seg_points(s_seg[warp])[(q0 & 15) + j] = make_float4(rrj[j][0], rrj[j][1], rrj[j][2], __int_as_float(segj[j]));
-      seg_add(s_seg[warp], lane);
+      seg_add<D>(s_seg[warp], lane);
     }
     if (!a.want_grad) continue;
     if (sl == 0) {
@@ -1525,7 +1531,7 @@ __global__ void __launch_bounds__(OT_THREADS, 2) k_out_loss_mma(const __grid_con
     }
     if (a.segpart) {   // uniform over the block
       if (lane < 16) seg_points(sseg)[lane] = make_float4(rr[0], rr[1], rr[2], __int_as_float(seg));
-      seg_add(sseg, lane);
+      seg_add<D>(sseg, lane);
     }
     if (a.want_grad) {
     __syncwarp();
