@@ -329,8 +329,9 @@ struct Acc2 {
 
 // Residual and seed for one point from its output jets U[c][r] (bias included).
 // k: the interior seed scale (k_pde, or the point's causal segment scale); rr: the
-// point's squared residual per equation (interior points); lacc (FP64, or FP32 for a
-// few points at a time) gathers the squared errors per loss term.
+// point's squared residual per equation (interior points; rounded on its own, whether or not
+// the caller uses it, so that the kernels' loss terms agree to the bit); lacc (FP64, or FP32
+// for a few points at a time) gathers the squared errors per loss term.
 template <int D, typename LT>
 __device__ __forceinline__ void point_residual(const OutArgs& a, int set, int64_t idx, float k, float U[3][4],
                                                float Ub[3][4], LT lacc[5], float rr[3]) {
@@ -344,20 +345,20 @@ __device__ __forceinline__ void point_residual(const OutArgs& a, int set, int64_
     if (a.pde == PINN_BURGERS_1D) {
       // rows [u, u_x, u_t, u_xx]
       const float r = U[0][2] + U[0][0] * U[0][1] - nu * U[0][3];
-      lacc[0] += (LT)r * r; rr[0] = r * r;
+      rr[0] = __fmul_rn(r, r); lacc[0] += rr[0];
       const float g2 = 2.f * k * r;
       Ub[0][0] = g2 * U[0][1]; Ub[0][1] = g2 * U[0][0]; Ub[0][2] = g2; Ub[0][3] = -nu * g2;
     } else if (a.pde == PINN_ADVECTION_1D) {
       // u_t + c u_x with c = nu (Sec. 4.1)
       const float r = fmaf(nu, U[0][1], U[0][2]);
-      lacc[0] += (LT)r * r; rr[0] = r * r;
+      rr[0] = __fmul_rn(r, r); lacc[0] += rr[0];
       const float g2 = 2.f * k * r;
       Ub[0][1] = nu * g2; Ub[0][2] = g2;
     } else if (a.pde == PINN_ALLEN_CAHN_1D) {
       // u_t - eps u_xx + 5 u^3 - 5 u with eps = nu (Sec. 4.2)
       const float u = U[0][0];
       const float r = U[0][2] - nu * U[0][3] + 5.f * u * (u * u - 1.f);
-      lacc[0] += (LT)r * r; rr[0] = r * r;
+      rr[0] = __fmul_rn(r, r); lacc[0] += rr[0];
       const float g2 = 2.f * k * r;
       Ub[0][0] = g2 * (15.f * u * u - 5.f); Ub[0][2] = g2; Ub[0][3] = -nu * g2;
     } else if (a.pde == PINN_NS_STEADY_2D) {
@@ -366,8 +367,8 @@ __device__ __forceinline__ void point_residual(const OutArgs& a, int set, int64_
       const float r1 = u * U[0][1] + v * U[0][2] + U[2 % D][1] - nu * U[0][3];
       const float r2 = u * U[1 % D][1] + v * U[1 % D][2] + U[2 % D][2] - nu * U[1 % D][3];
       const float r3 = U[0][1] + U[1 % D][2];
-      lacc[0] += (LT)r1 * r1; lacc[1] += (LT)r2 * r2; lacc[2] += (LT)r3 * r3;
-      rr[0] = r1 * r1; rr[1] = r2 * r2; rr[2] = r3 * r3;
+      rr[0] = __fmul_rn(r1, r1); rr[1] = __fmul_rn(r2, r2); rr[2] = __fmul_rn(r3, r3);
+      lacc[0] += rr[0]; lacc[1] += rr[1]; lacc[2] += rr[2];
       const float g1 = 2.f * k * r1, g2 = 2.f * k * r2, g3 = 2.f * k * r3;
       Ub[0][0] = g1 * U[0][1] + g2 * U[1 % D][1];
       Ub[1 % D][0] = g1 * U[0][2] + g2 * U[1 % D][2];
@@ -379,8 +380,8 @@ __device__ __forceinline__ void point_residual(const OutArgs& a, int set, int64_
       const float r1 = U[0][3] - (U[2 % D][1] - U[1 % D][2]);
       const float r2 = U[1 % D][3] + U[0][2];
       const float r3 = U[2 % D][3] - U[0][1];
-      lacc[0] += (LT)r1 * r1; lacc[1] += (LT)r2 * r2; lacc[2] += (LT)r3 * r3;
-      rr[0] = r1 * r1; rr[1] = r2 * r2; rr[2] = r3 * r3;
+      rr[0] = __fmul_rn(r1, r1); rr[1] = __fmul_rn(r2, r2); rr[2] = __fmul_rn(r3, r3);
+      lacc[0] += rr[0]; lacc[1] += rr[1]; lacc[2] += rr[2];
       const float g1 = 2.f * k * r1, g2 = 2.f * k * r2, g3 = 2.f * k * r3;
       Ub[0][3] = g1; Ub[2 % D][1] = -g1; Ub[1 % D][2] = g1;
       Ub[1 % D][3] = g2; Ub[0][2] = g2;
@@ -490,8 +491,12 @@ __device__ __forceinline__ double seg_total(float* sw0, int stride, int s, int k
 // lane = 8 * pg + sl: point group pg (4 consecutive points) and feature slice sl
 // (features sl, sl+8, ...).  The 8 slices of a point group combine their partial
 // outputs with three xor-shuffles; every slice then holds the group's outputs.
-template <typename T, int D, bool FAST, bool SINE>
-__global__ void __launch_bounds__(OUT_THREADS) k_out_loss(OutArgs a) {
+// SEG: the first pass of temporal causality (segment sums, no gradient), a kernel of its own: its
+// code in the others, behind a run-time test, cost them registers and up to 1.3 times the
+// time (FP32, 3 outputs, 1024 wide, loss at 5,000 points: 79 -> 102 us; without it 74).
+// BLOCKS: the blocks per SM that the registers are limited to, see out_loss_launch.
+template <typename T, int D, bool FAST, bool SINE, bool SEG, int BLOCKS>
+__global__ void __launch_bounds__(OUT_THREADS, BLOCKS) k_out_loss(OutArgs a) {
   // [d_out][w] weights, then [warps][d_out][w] dW accumulators, then [warps][w] bias
   // accumulators of the last hidden layer
   extern __shared__ float sW[];
@@ -510,8 +515,8 @@ __global__ void __launch_bounds__(OUT_THREADS) k_out_loss(OutArgs a) {
   const int64_t ntiles = a.NP / TILE_PTS;
   Acc2 acc[5];   // compensated FP32 running sums (FP64 is a slow pipe on this part)
   float dbo[3] = {0.f, 0.f, 0.f};                 // output bias gradient (value-row seeds)
-  __shared__ __align__(16) float s_seg[OUT_THREADS / 32][SEG_WORDS];   // causality: segment sums per warp
-  if (a.segpart) seg_clear(s_seg[warp], lane);
+  __shared__ __align__(16) float s_seg[SEG ? OUT_THREADS / 32 : 1][SEG ? SEG_WORDS : 4];   // segment sums per warp
+  if constexpr (SEG) seg_clear(s_seg[warp], lane);
   for (int64_t T0i = blockIdx.x; T0i < ntiles; T0i += gridDim.x) {
     const int64_t T0 = a.reverse ? ntiles - 1 - T0i : T0i;
     const int64_t cb = T0 * TILE_COLS + q0;        // column of row 0 of the first point
@@ -523,7 +528,7 @@ __global__ void __launch_bounds__(OUT_THREADS) k_out_loss(OutArgs a) {
       for (int c = 0; c < 3; ++c)
 #pragma unroll
         for (int r = 0; r < 4; ++r) U[j][c][r] = 0.f;
-#pragma unroll 2
+#pragma unroll 4
     for (int f = sl; f < w; f += 8) {
       const T* row = AL + toff(f, cb, w);
       float v[4][4];                               // [row][point]
@@ -579,14 +584,14 @@ __global__ void __launch_bounds__(OUT_THREADS) k_out_loss(OutArgs a) {
     }
     if (sl == 0)
       for (int i = 0; i < 5; ++i) acc[i].add(lacc[i]);
-    if (a.segpart) {   // uniform over the block
+    if constexpr (SEG) {
       if (sl == 0)
 #pragma unroll
         for (int j = 0; j < 4; ++j)
           seg_points(s_seg[warp])[(q0 & 15) + j] = make_float4(rrj[j][0], rrj[j][1], rrj[j][2], __int_as_float(segj[j]));
       seg_add<D>(s_seg[warp], lane);
     }
-    if (!a.want_grad) continue;
+    if (SEG || !a.want_grad) continue;
     if (sl == 0) {
 #pragma unroll
       for (int c = 0; c < D; ++c)
@@ -663,12 +668,12 @@ __global__ void __launch_bounds__(OUT_THREADS) k_out_loss(OutArgs a) {
     const double s = block_sum_d(acc[i].value(), sh);
     if (threadIdx.x == 0) a.losspart[(int64_t)blockIdx.x * 8 + i] = s;
   }
-  if (a.segpart) {
+  if constexpr (SEG) {
     __syncthreads();
     for (int i = threadIdx.x; i < CAUSAL_MAX * 4; i += blockDim.x)
       a.segpart[(int64_t)blockIdx.x * CAUSAL_MAX * 4 + i] = seg_total(s_seg[0], SEG_WORDS, i / 4, i % 4);
   }
-  if (!a.want_grad) return;
+  if (SEG || !a.want_grad) return;
   // block partials of the output layer's dW (warps summed in a fixed order) and bias
   __syncthreads();
   for (int i = threadIdx.x; i < D * w; i += blockDim.x) {
@@ -1639,15 +1644,31 @@ cudaError_t launch_out_loss_mma(pinn_handle* h, const OutArgs& a, int nblocks, c
 }
 
 
-template <typename T, int D, bool FAST, bool SINE>
-cudaError_t out_loss_launch(pinn_handle* h, const OutArgs& a, int nblocks, size_t smem, cudaStream_t st) {
-  auto kern = k_out_loss<T, D, FAST, SINE>;
+template <typename T, int D, bool FAST, bool SINE, bool SEG, int BLOCKS>
+cudaError_t out_loss_blocks_launch(pinn_handle* h, const OutArgs& a, int nblocks, size_t smem, cudaStream_t st) {
+  auto kern = k_out_loss<T, D, FAST, SINE, SEG, BLOCKS>;
   // weights + per-warp dW accumulators: up to 152 KB for 2048-wide, 3-output networks.  (Asked
   // for from the first byte: the 48 KB that need no asking hold the static memory as well.)
   const cudaError_t e = allow_smem(h, reinterpret_cast<const void*>(kern), smem);
   if (e != cudaSuccess) return e;
   kern<<<nblocks, OUT_THREADS, smem, st>>>(a);
   return cudaGetLastError();
+}
+
+// A block walks its tile's features with a few loads in flight, so latency bounds it, and the
+// blocks beside it hide that latency: as many per SM as registers allow (MANY) when there are enough
+// of them.  When all blocks are resident anyway, or shared memory lets no more in, the registers
+// of fewer (FEW) serve a block better.  One output, tanh (72 and 96 registers): 1024 wide at 5,000
+// points, loss 94 and 67 us, gradient 211 and 182; 256 wide at 60,000 points, gradient 202 and 262.
+// Three outputs, sine (128 and 168): 256 wide at 5,000 points, 71 and 66; BF16 at 60,000, 217 and 263.
+template <typename T, int D, bool FAST, bool SINE>
+cudaError_t out_loss_launch(pinn_handle* h, const OutArgs& a, int nblocks, size_t smem, cudaStream_t st) {
+  if (a.segpart) return out_loss_blocks_launch<T, D, FAST, SINE, true, D == 1 ? 5 : 4>(h, a, nblocks, smem, st);
+  constexpr int FEW = SINE ? 3 : D == 1 ? 5 : 4, MANY = SINE ? (D == 1 ? 3 : 4) : D == 1 ? 7 : 4;
+  constexpr size_t SM_BYTES = 228 * 1024, BLOCK_EXTRA = 1024 + 64;   // what the system and the static arrays take
+  const bool few = nblocks <= FEW * (int64_t)h->sm_count || SM_BYTES / (smem + BLOCK_EXTRA) < (size_t)MANY;
+  return few ? out_loss_blocks_launch<T, D, FAST, SINE, false, FEW>(h, a, nblocks, smem, st)
+             : out_loss_blocks_launch<T, D, FAST, SINE, false, MANY>(h, a, nblocks, smem, st);
 }
 
 cudaError_t launch_out_loss(pinn_handle* h, const OutArgs& a, int prec, int nblocks, cudaStream_t st) {

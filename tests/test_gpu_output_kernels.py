@@ -70,3 +70,39 @@ def test_register_output_kernel_other_widths(cuda_lib, widths):
     gt, gg = run_gpu(spec, p, B, b, Problem(0.0, 1.0, 1.0, 1.0), "bf16")
     rt, rg = run_oracle(spec, p, B, b, Problem(0.0, 1.0, 1.0, 1.0))
     assert_parity(gt, gg, rt, rg, TOL["bf16"], f"Maxwell {widths}", spec=spec)
+
+
+@pytest.mark.parametrize("pde,activation,n_res", [
+    ("burgers", "tanh", 48500), ("burgers", "tanh", 48700),   # 760 blocks: the line between the two register limits
+    ("ns", "sine", 29100), ("ns", "sine", 29200),             # 456 blocks
+    ("ns", "tanh", 200), ("burgers", "sine", 200),
+])
+def test_output_kernel_register_limits(cuda_lib, pde, activation, n_res):
+    """The CUDA-core output kernel on both sides of the rule that chooses its register limit."""
+    code, d_out = (PDE_BURGERS, 1) if pde == "burgers" else (PDE_NS, 3)
+    spec = NetSpec(code, 2, d_out, [12, 20], rwf=True)
+    spec.activation, spec.omega0 = activation, 1.5
+    p, prob = init_params(spec, 61, 0.2), Problem(0.02, 0.3, 2.0, 5.0)
+    b = make_batch(code, n_res, 10 if d_out == 1 else 0, 20, 62, 63)
+    gt, gg = run_gpu(spec, p, None, b, prob, "fp32")
+    rt, rg = run_oracle(spec, p, None, b, prob, chunk=16384)
+    assert_parity(gt, gg, rt, rg, TOL["fp32"], f"{pde} {activation} {n_res}", spec=spec)
+
+
+@pytest.mark.parametrize("width,precision", [(13, "fp32"), (64, "bf16"), (288, "bf16"), (600, "bf16")])
+def test_one_causal_segment_without_decay_is_the_plain_loss(cuda_lib, width, precision):
+    """With one segment and eps = 0 the causal pass sums the plain loss (the plain kernels add up to
+    four points in FP32 first: 3 roundings), and the gradient is the plain one bit for bit."""
+    import torch
+    from paper_2604_15645_gb300 import api
+    spec = NetSpec(PDE_BURGERS, 2, 1, [16, width])
+    params = torch.tensor(init_params(spec, 51, 0.2), device="cuda")
+    db, prob = api.DeviceBatch.from_host(make_batch(PDE_BURGERS, 5000, 40, 30, 52, 53)), api.make_problem(0.05, 0.7, 0.5, 2.0)
+    plain, causal = (api.PinnNet.from_spec(spec, precision) for _ in range(2))
+    causal.set_causal(1, 0.0)
+    t0, g0 = plain.loss_grad(params, db, prob)
+    t1, g1 = causal.loss_grad(params, db, prob)
+    torch.cuda.synchronize()
+    assert plain.status_poll() == 0 and causal.status_poll() == 0
+    assert torch.allclose(t0, t1, rtol=2.0 ** -22, atol=0.0)
+    assert torch.equal(g0, g1)
