@@ -261,3 +261,33 @@ def test_single_gemm_layer(cuda_lib, widths, ff, n_res):
     torch.cuda.synchronize()
     assert net.status_poll() == 0 and multi.status_poll() == 0
     assert torch.equal(terms, ref[0]) and torch.equal(grad, g) and torch.equal(loss, terms)
+
+
+@pytest.mark.parametrize("pde", [PDE_BURGERS, PDE_NS, PDE_MAXWELL])
+@pytest.mark.parametrize("width", [64, 320])   # every layer in one kernel; layer by layer
+def test_packed_forward_rule_matches_the_scalar_one(cuda_lib, pde, width):
+    """The tensor-core epilogues' packed tanh-jet rule against the scalar rule of the CUDA-core
+    kernels, on layers whose products and sums are exact in both (one power of two per row): the
+    same losses bit for bit."""
+    from paper_2604_15645_gb300 import _lib, api
+    from parity_blocks import param_blocks
+    d_in, d_out = (3, 3) if pde == PDE_MAXWELL else (2, 1 if pde == PDE_BURGERS else 3)
+    spec = NetSpec(pde, d_in, d_out, [width] * 3)
+    p = init_params(spec, 31, 0.2).astype(np.float32)
+    rng = np.random.default_rng(32)
+    blocks = {n: (s, e) for n, s, e in param_blocks(spec)}
+    for name in ("V2", "V3"):
+        W = np.zeros((width, width), np.float32)
+        W[np.arange(width), rng.permutation(width)] = 2.0 ** rng.integers(-2, 5, width) * rng.choice([-1, 1], width)
+        p[slice(*blocks[name])] = W.ravel()
+    db = api.DeviceBatch.from_host(make_batch(pde, 6000, 0 if pde == PDE_NS else 50, 60, 33, 34))
+    prob, params = api.make_problem(0.02, 0.5, 1.0, 2.0), torch.tensor(p, device="cuda")
+    res = []
+    for flags in (0, _lib.PINN_FLAG_CUDA_CORES):
+        net = api.PinnNet.from_spec(spec, "bf16")
+        _lib.pinn_destroy(net.h)
+        net.h = _lib.pinn_create(_lib.make_spec(pde, spec.widths, 0, False, _lib.PRECISIONS["bf16"], flags))
+        res.append(net.loss(params, db, prob).clone())
+        torch.cuda.synchronize()
+        assert net.status_poll() == 0
+    assert torch.equal(res[0], res[1])
