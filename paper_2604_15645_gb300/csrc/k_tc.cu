@@ -136,15 +136,18 @@ struct GroupShare {
 struct PairGrid : SingleGrid {
   static constexpr bool PAIR = true;
 };
+// After an abort: MMAs that are still on their way read shared memory and write tensor memory
+// (and, in a pair, copies and arrivals reach the other CTA).  No barrier tells when, but they
+// take microseconds: wait them out (1 ms) before any of that memory is given back.
+__device__ __forceinline__ void abort_settle() {
+  const uint64_t t0 = gtimer();
+  while (gtimer() - t0 < 1000000ull) {}
+}
 // Last step of a CTA of a pair: the other one arrives at this one's barriers and its MMAs
-// read this one's shared memory, so neither leaves before both are done.  (After an abort
-// MMAs, copies and arrivals that are still on their way take microseconds: wait them out.)
+// read this one's shared memory, so neither leaves before both are done.
 __device__ __forceinline__ void pair_leave(volatile int* abort_flag) {
   cluster_sync();
-  if (threadIdx.x == 0 && *abort_flag) {
-    const uint64_t t0 = gtimer();
-    while (gtimer() - t0 < 1000000ull) {}
-  }
+  if (threadIdx.x == 0 && *abort_flag) abort_settle();
   cluster_sync();
 }
 
@@ -903,7 +906,7 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA, const CUte
     }
   }
 
-  // ---- teardown: wait (bounded) for copies still in flight, free TMEM ----------------
+  // ---- teardown: wait (bounded) for copies and MMAs still in flight, free TMEM ----------------
   __syncthreads();
   if (threadIdx.x == 0 && *abort_flag) {
     for (int s = 0; s < C::STAGES; ++s) {
@@ -913,6 +916,7 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap* mapA, const CUte
         while (!mbar_try(&full[s], (uint32_t)(f - 1)) && gtimer() - t0 < WAIT_NS) {}
       }
     }
+    if (!PAIR) abort_settle();
   }
   tc_fence_before();
   __syncthreads();
@@ -1619,7 +1623,7 @@ __device__ __forceinline__ void tc_adjdw_body(const CUtensorMap* mapW, const CUt
     }
   }
 
-  // ---- teardown: wait (bounded) for copies still in flight, free TMEM ----------------
+  // ---- teardown: wait (bounded) for copies and MMAs still in flight, free TMEM ----------------
   __syncthreads();
   if (threadIdx.x == 0 && *abort_flag) {
     for (int s = 0; s < FZ_STAGES; ++s) {
@@ -1636,6 +1640,7 @@ __device__ __forceinline__ void tc_adjdw_body(const CUtensorMap* mapW, const CUt
         while (!mbar_try(&a_full[b], (uint32_t)(f - 1)) && gtimer() - t0 < WAIT_NS) {}
       }
     }
+    abort_settle();
   }
   tc_fence_before();
   __syncthreads();
@@ -2108,7 +2113,7 @@ __global__ void __launch_bounds__(FF_NT, 1) k_tc_fwd_all(const __grid_constant__
         }
   }
 
-  // ---- teardown: wait (bounded) for copies still in flight, free TMEM ----------------
+  // ---- teardown: wait (bounded) for copies and MMAs still in flight, free TMEM ----------------
   __syncthreads();
   if (threadIdx.x == 0 && *abort_flag) {
     auto drain = [&](uint64_t* bar, int f) {
@@ -2118,6 +2123,7 @@ __global__ void __launch_bounds__(FF_NT, 1) k_tc_fwd_all(const __grid_constant__
     };
     for (int i = 0; i < FF_WSTAGES; ++i) drain(&wfull[i], w_inflight[i]);
     for (int i = 0; i < 4; ++i) drain(&afull[i], a_inflight[i]);
+    abort_settle();
   }
   tc_fence_before();
   __syncthreads();
