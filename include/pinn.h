@@ -395,6 +395,14 @@ PINN_API pinn_status pinn_tc_selftest(int kind, int M, int N, int K, const void*
 PINN_API pinn_status pinn_debug_wait_expiry(pinn_handle* h, int M, int N, int K, const void* d_A, const void* d_B,
                                             float* d_D, int64_t wait_us, void* stream);
 
+/* Test hook for failure detection, with no counterpart in the paper: while wait_us > 0
+ * (up to 2,000,000), the tcgen05 kernels of every pass of h (loss, gradient; single and
+ * paired CTAs, the one-kernel forward, the fused adjoint) have their MMA-issuing thread
+ * first wait on an mbarrier that no thread ever arrives on, with every wait of these kernels
+ * bounded by wait_us microseconds.  They end as in pinn_debug_wait_expiry; the pass's results are
+ * undefined and pinn_status_poll(h) reports PINN_ERR_TIMEOUT.  0 switches it off. */
+PINN_API pinn_status pinn_debug_stall(pinn_handle* h, int64_t wait_us);
+
 /* ---- many independent networks in one training step --------------------------------
  * A pinn_multi holds one network handle per spec (uneven widths, depths and point
  * counts allowed).  pinn_multi_train_step runs, for every network, the loss and

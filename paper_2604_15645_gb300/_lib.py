@@ -31,7 +31,7 @@ EXPORTS = ["pinn_create", "pinn_destroy", "pinn_param_count", "pinn_workspace_by
            "pinn_loss_grad_terms", "pinn_loss_balance", "pinn_set_causal", "pinn_causal_weights",
            "pinn_lbfgs_create", "pinn_lbfgs_destroy", "pinn_lbfgs_reset", "pinn_lbfgs_step", "pinn_lbfgs_direction",
            "pinn_lbfgs_push_pair", "pinn_set_activation", "pinn_set_periodic", "pinn_loss_grad_ff",
-           "pinn_set_graph", "pinn_set_global_counts", "pinn_graph_held", "pinn_debug_wait_expiry",
+           "pinn_set_graph", "pinn_set_global_counts", "pinn_graph_held", "pinn_debug_wait_expiry", "pinn_debug_stall",
            "pinn_layer_engines", "pinn_multi_set_config", "pinn_multi_get_config", "pinn_multi_set_grouped",
            "pinn_multi_get_grouped"]
 PINN_ACT_TANH, PINN_ACT_SINE = 0, 1
@@ -123,6 +123,7 @@ def load(path: str = LIB_PATH):
     lib.pinn_set_activation.argtypes = [H, C.c_int, C.c_double]
     lib.pinn_set_graph.argtypes = [H, C.c_int]
     lib.pinn_graph_held.argtypes = [H, C.POINTER(C.c_int32)]
+    lib.pinn_debug_stall.argtypes = [H, C.c_int64]
     lib.pinn_debug_wait_expiry.argtypes = [H, C.c_int, C.c_int, C.c_int, C.c_void_p, C.c_void_p, C.c_void_p,
                                            C.c_int64, C.c_void_p]
     lib.pinn_set_global_counts.argtypes = [H, C.c_int64, C.c_int64, C.c_int64]
@@ -226,6 +227,10 @@ def pinn_graph_held(h: int) -> bool:
     held = C.c_int32()
     check(load().pinn_graph_held(h, C.byref(held)), h)
     return bool(held.value)
+
+
+def pinn_debug_stall(h, wait_us):
+    check(load().pinn_debug_stall(h, wait_us), h)
 
 
 def pinn_debug_wait_expiry(h, M, N, K, d_A, d_B, d_D, wait_us, stream):

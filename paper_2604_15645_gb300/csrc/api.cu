@@ -738,6 +738,7 @@ pinn_status run_graphed(pinn_handle* h, int kind, const pinn_problem* prob, cons
   k.ff_B = h->ff_B; k.periodic = h->periodic ? 1 : 0;
   for (int i = 0; i < 3; ++i) k.periods[i] = h->periods[i];
   k.stream = stream;
+  k.stall_ns = h->stall_ns;
   if (!h->graph_exec || memcmp(&k, &h->graph_key, sizeof(k)) != 0) {
     drop_graph(h);
     if (cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeRelaxed) != cudaSuccess) {

@@ -1134,7 +1134,7 @@ int tc_dw_splits(const pinn_handle* h, int fout, int fin, int64_t NC) {
 
 namespace {
 
-TcParams base_params(int M, int N, int K, int64_t NC, int kblock, int* status) {
+TcParams base_params(const pinn_handle* h, int M, int N, int K, int64_t NC, int kblock, int* status) {
   TcParams p{};
   p.M = M; p.N = N; p.K = K; p.NC = NC;
   p.m_tiles = (M + BM - 1) / BM;
@@ -1142,8 +1142,8 @@ TcParams base_params(int M, int N, int K, int64_t NC, int kblock, int* status) {
   p.k_iters = (K + kblock - 1) / kblock;
   p.nsplit = 1; p.kps = p.k_iters;
   p.status = status;
-  p.wait_ns = WAIT_NS;
-  p.stall = 0;
+  p.wait_ns = h->stall_ns ? h->stall_ns : WAIT_NS;
+  p.stall = h->stall_ns ? 1 : 0;
   return p;
 }
 
@@ -1173,7 +1173,7 @@ pinn_status fwd_impl(pinn_handle* h, const void* W, const void* Wlo, const void*
     if (!make_map3(&mlo, Alo, false, TILE_PTS, fin, nt, C::BOXN, C::BKE))
       return map_err(h, "forward value-row low half");
   }
-  TcParams p = base_params(fout, (int)NC, fin, NC, C::BKE, h->d_status);
+  TcParams p = base_params(h, fout, (int)NC, fin, NC, C::BKE, h->d_status);
   p.e = e;
   p.wlo_values_only = (!TF32 && (h->spec.flags & PINN_FLAG_BF16_VALUE_SPLIT)) ? 1 : 0;
   const int grid = grid_for(h, p.m_tiles * p.n_tiles);
@@ -1220,7 +1220,7 @@ pinn_status adj_impl(pinn_handle* h, const void* WT, const void* WTlo, const voi
     if (!make_map3(&mb, Zbar, false, TILE_COLS, fout, (uint64_t)(NC / TILE_COLS), C::BOXN, C::BKE))
       return map_err(h, "adjoint input");
   }
-  TcParams p = base_params(fin, (int)NC, fout, NC, C::BKE, h->d_status);
+  TcParams p = base_params(h, fin, (int)NC, fout, NC, C::BKE, h->d_status);
   p.e = e;
   const int grid = grid_for(h, p.m_tiles * p.n_tiles);
   return launch<TF32, TC_ADJ, SPLIT, !TF32>(h, ma, ma2, mb, mb, p, grid, st);
@@ -1235,7 +1235,7 @@ pinn_status dw_impl(pinn_handle* h, const void* Zbar, const void* A, int fout, i
   const uint64_t nt = (uint64_t)(NC / TILE_COLS);
   if (!make_map3(&ma, Zbar, TF32, TILE_COLS, fout, nt, C::BKE, BM)) return map_err(h, "weight-gradient adjoint");
   if (!make_map3(&mb, A, TF32, TILE_COLS, fin, nt, C::BKE, BN)) return map_err(h, "weight-gradient activations");
-  TcParams p = base_params(fout, fin, (int)NC, NC, C::BKE, h->d_status);
+  TcParams p = base_params(h, fout, fin, (int)NC, NC, C::BKE, h->d_status);
   if (two) p.m_tiles = (fout + 2 * BM - 1) / (2 * BM);
   p.nsplit = nsplit;
   p.kps = (p.k_iters + nsplit - 1) / nsplit;
@@ -1339,7 +1339,8 @@ __device__ __forceinline__ void tc_adjdw_body(const CUtensorMap* mapW, const CUt
   uint64_t* a_full = acc_empty + ACC;
   uint64_t* z_done = a_full + FZ_ABUF;
   uint64_t* dw_full = z_done + FZ_ABUF;
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(dw_full + 1);
+  uint64_t* never = dw_full + 1;                 // test hook (p.stall): no thread arrives on it
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(never + 1);
   volatile int* inflight = abort_flag + 1;              // [FZ_STAGES]
   volatile int* a_inflight = inflight + FZ_STAGES;      // [FZ_ABUF]
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(const_cast<int*>(a_inflight + FZ_ABUF));
@@ -1361,6 +1362,7 @@ __device__ __forceinline__ void tc_adjdw_body(const CUtensorMap* mapW, const CUt
       mbar_init(&acc_empty[b], FZ_EPI);
     }
     mbar_init(dw_full, 1);
+    mbar_init(never, 1);
     *abort_flag = 0;
     fence_mbar_init();
   }
@@ -1468,7 +1470,7 @@ __device__ __forceinline__ void tc_adjdw_body(const CUtensorMap* mapW, const CUt
       int stage = 0;
       uint32_t phase = 0;
       int local = 0;
-      bool ok = true;
+      bool ok = !p.stall || mbar_wait(never, 0, abort_flag, p.status, p.wait_ns);
       for (int t = grid.bx(); t < total && !*abort_flag && ok; t += grid.gdim(), ++local) {
         const int ab = local % FZ_ABUF, buf = local % ACC;
         const uint32_t d_adj = tmem_base + buf * BN;
@@ -1711,7 +1713,7 @@ pinn_status adj_staged(pinn_handle* h, const void* WT, const void* Zbar, int fin
   if (!make_map3(&ma, e.ain, false, TILE_COLS, fin, nt, 64, BM)) return map_err(h, "adjoint activations");
   mo = ma;
   if (e.out && !make_map3(&mo, e.out, false, TILE_COLS, fin, nt, 64, BM)) return map_err(h, "adjoint output");
-  TcParams p = base_params(fin, (int)NC, fout, NC, 64, h->d_status);
+  TcParams p = base_params(h, fin, (int)NC, fout, NC, 64, h->d_status);
   p.e = e;
   return launch_adjdw<false>(h, mw, mz, ma, mo, p, grid_for(h, p.m_tiles * p.n_tiles), st);
 }
@@ -1737,7 +1739,7 @@ pinn_status tc_gemm_adjdw(pinn_handle* h, const void* WT, const void* Zbar, cons
   if (!make_map3(&mz, Zbar, false, TILE_COLS, fout, nt, 64, 64)) return map_err(h, "fused adjoint input");
   if (!make_map3(&ma, Ain, false, TILE_COLS, fin, nt, 64, BM)) return map_err(h, "fused adjoint activations");
   mo = ma;   // (not used: this form stores from registers)
-  TcParams p = base_params(fin, (int)NC, fout, NC, 64, h->d_status);
+  TcParams p = base_params(h, fin, (int)NC, fout, NC, 64, h->d_status);
   p.e = e;
   p.out32 = dwpart;
   const int grid = adjdw_grid(h, fin, NC);
@@ -1808,6 +1810,7 @@ struct FwdAllParams {
   int store;                                 // write A_l of the layers below the last
   int* status;
   uint64_t wait_ns;
+  int stall;                                 // test hook, as in TcParams
 };
 
 template <bool M2>
@@ -1826,7 +1829,8 @@ __global__ void __launch_bounds__(FF_NT, 1) k_tc_fwd_all(const __grid_constant__
   uint64_t* accr = accf + 2;                      // [2]
   uint64_t* done = accr + 2;                      // [2]
   uint64_t* sread = done + 2;                     // [2]
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(sread + 2);
+  uint64_t* never = sread + 2;                    // test hook (p.stall): no thread arrives on it
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(never + 1);
   volatile int* w_inflight = abort_flag + 1;      // [FF_WSTAGES]
   volatile int* a_inflight = w_inflight + FF_WSTAGES;   // [4]
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(const_cast<int*>(a_inflight + 4));
@@ -1846,6 +1850,7 @@ __global__ void __launch_bounds__(FF_NT, 1) k_tc_fwd_all(const __grid_constant__
       mbar_init(&done[i], FZ_EPI);
       mbar_init(&sread[i], 1);
     }
+    mbar_init(never, 1);
     *abort_flag = 0;
     fence_mbar_init();
   }
@@ -1940,7 +1945,7 @@ __global__ void __launch_bounds__(FF_NT, 1) k_tc_fwd_all(const __grid_constant__
       uint32_t ph = 0, round = 0;
       int jobs[2] = {0, 0};                       // jobs issued per accumulator
       int written[2] = {0, 0};                    // those of layers below the last
-      bool ok = true;
+      bool ok = !p.stall || mbar_wait(never, 0, abort_flag, p.status, p.wait_ns);
       auto wait = [&](uint64_t* bar, uint32_t par) {
         if (ok) ok = mbar_wait(bar, par, abort_flag, p.status, p.wait_ns);
         return ok;
@@ -2163,7 +2168,8 @@ pinn_status tc_gemm_fwd_all(pinn_handle* h, const TcFwdLayer* layers, int n, con
   p.store = store && n > 1;   // (a single layer leaves through the epilogue)
   p.wlo_values_only = (h->spec.flags & PINN_FLAG_BF16_VALUE_SPLIT) ? 1 : 0;
   p.status = h->d_status;
-  p.wait_ns = WAIT_NS;
+  p.wait_ns = h->stall_ns ? h->stall_ns : WAIT_NS;
+  p.stall = h->stall_ns ? 1 : 0;
   auto kern = m2 ? k_tc_fwd_all<true> : k_tc_fwd_all<false>;
   const pinn_status s = reserve_smem(h, kern, FF_SMEM, "fused forward kernel");
   if (s) return s;
@@ -2263,10 +2269,9 @@ pinn_status selftest_impl(pinn_handle* h, int layout, int M, int N, int K, const
     if (!make_map(&ma, d_A, TF32, K, M, C::BKE, BM) || !make_map(&ma2, d_A2 ? d_A2 : d_A, TF32, K, M, C::BKE, BM) ||
         !make_map3(&mb, d_B, TF32, TILE_COLS, K, N / TILE_COLS, C::BOXN, C::BKE))
       return PINN_ERR_CUDA;
-    TcParams p = base_params(M, N, K, N, C::BKE, status);
+    TcParams p = base_params(h, M, N, K, N, C::BKE, status);
     p.out32 = d_D;
-    if (wait_ns) p.wait_ns = wait_ns;
-    p.stall = stall;
+    if (stall) { p.wait_ns = wait_ns; p.stall = 1; }
     const int grid = grid_for(h, p.m_tiles * p.n_tiles);
     if (d_A2) return launch<TF32, TC_STORE, true>(h, ma, ma2, mb, mb, p, grid, st);
     return launch<TF32, TC_STORE, false>(h, ma, ma, mb, mb, p, grid, st);
@@ -2276,7 +2281,7 @@ pinn_status selftest_impl(pinn_handle* h, int layout, int M, int N, int K, const
   if (!make_map3(&ma, d_A, TF32, TILE_COLS, M, K / TILE_COLS, C::BKE, BM) ||
       !make_map3(&mb, d_B, TF32, TILE_COLS, N, K / TILE_COLS, C::BKE, BN))
     return PINN_ERR_CUDA;
-  TcParams p = base_params(M, N, K, N, C::BKE, status);
+  TcParams p = base_params(h, M, N, K, N, C::BKE, status);
   p.out32 = d_D;
   return launch<TF32, TC_DW, false>(h, ma, ma, mb, mb, p, grid_for(h, p.m_tiles * p.n_tiles), st);
 }
@@ -2313,6 +2318,12 @@ extern "C" PINN_API pinn_status pinn_tc_selftest(int kind, int M, int N, int K, 
   }
   cudaFree(status);
   return r;
+}
+
+extern "C" PINN_API pinn_status pinn_debug_stall(pinn_handle* h, int64_t wait_us) {
+  if (!h || wait_us < 0 || wait_us > 2000000) return PINN_ERR_INVALID_ARG;
+  h->stall_ns = (uint64_t)wait_us * 1000ull;
+  return PINN_OK;
 }
 
 extern "C" PINN_API pinn_status pinn_debug_wait_expiry(pinn_handle* h, int M, int N, int K, const void* d_A,
