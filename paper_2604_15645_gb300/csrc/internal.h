@@ -112,7 +112,7 @@ struct pinn_handle {
   int act = PINN_ACT_TANH;   // hidden activation; sine keeps Z and runs on CUDA cores
   pinn::TcBatch* tc_batch = nullptr;   // set: tensor-core GEMMs are collected for a grouped launch
   float omega0 = 1.f;
-  uint64_t stall_ns = 0;     // test hook (pinn_debug_stall): stall the MMA issuers, with this bound on every wait
+  uint64_t stall_ns = 0;     // test hook (pinn_debug_stall): an arrival that never comes, and this bound on every wait
   char err[512] = {0};
   // phase profiler (pinn_set_profiling)
   bool prof = false;

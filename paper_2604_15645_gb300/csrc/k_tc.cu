@@ -85,7 +85,8 @@ struct TcParams {
   int* status;
   int wlo_values_only; // forward: W_lo . B on the 64 value columns only (PINN_FLAG_BF16_VALUE_SPLIT)
   uint64_t wait_ns;    // bound on every mbarrier wait (WAIT_NS)
-  int stall;           // test hook: the MMA issuer first waits on a barrier nothing arrives on
+  int stall;           // test hook: the MMA issuer first waits on a barrier nothing arrives on (fused
+                       // adjoint: no activation tile comes)
 };
 
 // One GEMM of a grouped launch: its tensor maps (the GEMM kernel's four, or the fused
@@ -1339,8 +1340,7 @@ __device__ __forceinline__ void tc_adjdw_body(const CUtensorMap* mapW, const CUt
   uint64_t* a_full = acc_empty + ACC;
   uint64_t* z_done = a_full + FZ_ABUF;
   uint64_t* dw_full = z_done + FZ_ABUF;
-  uint64_t* never = dw_full + 1;                 // test hook (p.stall): no thread arrives on it
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(never + 1);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(dw_full + 1);
   volatile int* inflight = abort_flag + 1;              // [FZ_STAGES]
   volatile int* a_inflight = inflight + FZ_STAGES;      // [FZ_ABUF]
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(const_cast<int*>(a_inflight + FZ_ABUF));
@@ -1362,7 +1362,6 @@ __device__ __forceinline__ void tc_adjdw_body(const CUtensorMap* mapW, const CUt
       mbar_init(&acc_empty[b], FZ_EPI);
     }
     mbar_init(dw_full, 1);
-    mbar_init(never, 1);
     *abort_flag = 0;
     fence_mbar_init();
   }
@@ -1435,7 +1434,9 @@ __device__ __forceinline__ void tc_adjdw_body(const CUtensorMap* mapW, const CUt
         t_out += grid.gdim();
         ++out;
       };
-      for (int t = grid.bx(); t < total && ok && !*abort_flag; t += grid.gdim(), ++in) {
+      // (test hook, single launches: with p.stall no tile comes, and the waits for it expire)
+      const bool stall = std::is_same<Grid, SingleGrid>::value && p.stall;
+      for (int t = stall ? total : grid.bx(); t < total && ok && !*abort_flag; t += grid.gdim(), ++in) {
         int mb, nb;
         coords(t, mb, nb);
         const int ab = in % FZ_ABUF;
@@ -1470,7 +1471,7 @@ __device__ __forceinline__ void tc_adjdw_body(const CUtensorMap* mapW, const CUt
       int stage = 0;
       uint32_t phase = 0;
       int local = 0;
-      bool ok = !p.stall || mbar_wait(never, 0, abort_flag, p.status, p.wait_ns);
+      bool ok = true;
       for (int t = grid.bx(); t < total && !*abort_flag && ok; t += grid.gdim(), ++local) {
         const int ab = local % FZ_ABUF, buf = local % ACC;
         const uint32_t d_adj = tmem_base + buf * BN;
@@ -1810,7 +1811,7 @@ struct FwdAllParams {
   int store;                                 // write A_l of the layers below the last
   int* status;
   uint64_t wait_ns;
-  int stall;                                 // test hook, as in TcParams
+  int stall;                                 // test hook: the weight producer brings nothing
 };
 
 template <bool M2>
@@ -1829,8 +1830,7 @@ __global__ void __launch_bounds__(FF_NT, 1) k_tc_fwd_all(const __grid_constant__
   uint64_t* accr = accf + 2;                      // [2]
   uint64_t* done = accr + 2;                      // [2]
   uint64_t* sread = done + 2;                     // [2]
-  uint64_t* never = sread + 2;                    // test hook (p.stall): no thread arrives on it
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(never + 1);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(sread + 2);
   volatile int* w_inflight = abort_flag + 1;      // [FF_WSTAGES]
   volatile int* a_inflight = w_inflight + FF_WSTAGES;   // [4]
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(const_cast<int*>(a_inflight + 4));
@@ -1850,7 +1850,6 @@ __global__ void __launch_bounds__(FF_NT, 1) k_tc_fwd_all(const __grid_constant__
       mbar_init(&done[i], FZ_EPI);
       mbar_init(&sread[i], 1);
     }
-    mbar_init(never, 1);
     *abort_flag = 0;
     fence_mbar_init();
   }
@@ -1883,7 +1882,8 @@ __global__ void __launch_bounds__(FF_NT, 1) k_tc_fwd_all(const __grid_constant__
       int st = 0;
       uint32_t ph = 0;
       bool ok = true;
-      for (int base = blockIdx.x; base < p.ntiles && ok; base += SLOTS * g)
+      // (test hook: with p.stall it brings nothing, and the waits for its weights expire)
+      for (int base = p.stall ? p.ntiles : blockIdx.x; base < p.ntiles && ok; base += SLOTS * g)
         for (int l = 0; l < L && ok; ++l) {
           const int nk = (p.fin[l] + 63) >> 6;
           for (int hh = 0; hh < 2 * HALVES && ok; ++hh) {
@@ -1945,7 +1945,7 @@ __global__ void __launch_bounds__(FF_NT, 1) k_tc_fwd_all(const __grid_constant__
       uint32_t ph = 0, round = 0;
       int jobs[2] = {0, 0};                       // jobs issued per accumulator
       int written[2] = {0, 0};                    // those of layers below the last
-      bool ok = !p.stall || mbar_wait(never, 0, abort_flag, p.status, p.wait_ns);
+      bool ok = true;
       auto wait = [&](uint64_t* bar, uint32_t par) {
         if (ok) ok = mbar_wait(bar, par, abort_flag, p.status, p.wait_ns);
         return ok;
@@ -2165,7 +2165,7 @@ pinn_status tc_gemm_fwd_all(pinn_handle* h, const TcFwdLayer* layers, int n, con
   p.a_last = reinterpret_cast<__nv_bfloat16*>(layers[n - 1].out);
   p.alo_last = reinterpret_cast<__nv_bfloat16*>(alo_last);
   p.layers = n; p.ntiles = (int)nt; p.reverse = reverse; p.jet_mode = jet_mode;
-  p.store = store && n > 1;   // (a single layer leaves through the epilogue)
+  p.store = store;
   p.wlo_values_only = (h->spec.flags & PINN_FLAG_BF16_VALUE_SPLIT) ? 1 : 0;
   p.status = h->d_status;
   p.wait_ns = h->stall_ns ? h->stall_ns : WAIT_NS;

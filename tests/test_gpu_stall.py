@@ -1,6 +1,6 @@
-"""Failure detection in the kernels of a whole pass, without a GPU fault: pinn_debug_stall makes
-the MMA issuers of a handle's tcgen05 kernels wait on a barrier that nothing arrives on, under a
-1 ms bound.  Every kernel of the pass must end through its abort path, the host must read
+"""Failure detection in the kernels of a whole pass, without a GPU fault: pinn_debug_stall launches
+a handle's tcgen05 kernels with an arrival that never comes, under a 1 ms bound on every wait.
+Every kernel of the pass must end through its abort path, the host must read
 PINN_ERR_TIMEOUT, and the context must stay usable: the same call without the stall gives
 the bits it gave before."""
 import pytest
