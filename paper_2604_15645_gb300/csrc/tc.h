@@ -30,8 +30,8 @@ int tc_dw_splits(const pinn_handle* h, int fout, int fin, int64_t NC);
 //         the epilogue also writes e.out_pm (point-major A_l) when set.
 pinn_status tc_gemm_fwd(pinn_handle* h, const void* W, const void* Wlo, const void* A, const void* Alo, int fout,
                         int fin, int64_t NC, const EpiArgs& e, cudaStream_t st);
-// Every hidden GEMM layer of the forward in one launch (BF16 tanh networks whose hidden
-// widths and first fan-in are at most 256), bitwise the per-layer launches.  `in` / `in_lo`
+// Every hidden GEMM layer of the forward in one launch (BF16 tanh networks of two or more such
+// layers whose widths and first fan-in are at most 256), bitwise the per-layer launches.  `in` / `in_lo`
 // are the first layer's input jets and low half; each layer's out receives A_l (with
 // store = 0, a loss-only call, only the last layer's does), alo_last the low half of A_L.
 struct TcFwdLayer {

@@ -291,3 +291,36 @@ def test_packed_forward_rule_matches_the_scalar_one(cuda_lib, pde, width):
         torch.cuda.synchronize()
         assert net.status_poll() == 0
     assert torch.equal(res[0], res[1])
+
+
+@pytest.mark.parametrize("n_res", [38879, 38880])
+def test_fp32_weight_gradient_forms(cuda_lib, n_res):
+    """One 64 x 64 weight-gradient tile in 608 splits: 256 columns each (the last size of the
+    four-column form) and 288 (the first of the eight-column one), on 152 SMs."""
+    spec = NetSpec(PDE_NS, 2, 3, [64], ff_m=32, ff_sigma=1.0, rwf=True)
+    _parity(spec, n_res, 0, 33, "fp32", f"fp32 weight gradient, {n_res} points")
+
+
+@pytest.mark.parametrize("pde,widths,ff", [(PDE_NS, [136, 24, 200], 8), (PDE_BURGERS, [72, 264], 0)])
+@pytest.mark.parametrize("n_res", [1, 7000])
+def test_tf32_edges_per_block(cuda_lib, pde, widths, ff, n_res):
+    """The TF32 epilogues at the precision's stated tolerance, per loss term and per block of the
+    gradient."""
+    spec = NetSpec(pde, 2, 1 if pde == PDE_BURGERS else 3, widths, ff_m=ff, ff_sigma=1.0)
+    p, B, prob = init_params(spec, 81, 0.2), ff_matrix(spec, 82), Problem(0.02, 0.3, 2.0, 5.0)
+    b = make_batch(pde, n_res, 30, 20, 83, 84)
+    gt, gg = run_gpu(spec, p, B, b, prob, "tf32")
+    rt, rg = run_oracle(spec, p, B, b, prob, chunk=4096)
+    assert_parity(gt, gg, rt, rg, TOL["tf32"], f"tf32 {widths} {n_res}", spec=spec)
+
+
+@pytest.mark.parametrize("pde,widths,ff", [
+    (PDE_BURGERS, [264, 272], 0), (PDE_NS, [512, 304, 264], 16), (PDE_MAXWELL, [40, 1024, 16], 0)])
+def test_wide_layer_edges_per_block(cuda_lib, pde, widths, ff):
+    """Layers above 256 wide, full split of the weights: per loss term and per block of the gradient."""
+    spec = NetSpec(pde, 3 if pde == PDE_MAXWELL else 2, 1 if pde == PDE_BURGERS else 3, widths, ff_m=ff, ff_sigma=1.0)
+    p, B, prob = init_params(spec, 95, 0.2), ff_matrix(spec, 96), Problem(0.02, 0.3, 2.0, 5.0)
+    b = make_batch(pde, 7000, 30, 20, 97, 98)
+    gt, gg = run_gpu(spec, p, B, b, prob, "bf16")
+    rt, rg = run_oracle(spec, p, B, b, prob, chunk=4096)
+    assert_parity(gt, gg, rt, rg, TOL["bf16"], f"bf16 {widths}", spec=spec)
