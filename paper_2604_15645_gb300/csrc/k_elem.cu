@@ -1656,17 +1656,20 @@ cudaError_t out_loss_blocks_launch(pinn_handle* h, const OutArgs& a, int nblocks
 }
 
 // A block walks its tile's features with a few loads in flight, so latency bounds it, and the
-// blocks beside it hide that latency: as many per SM as registers allow (MANY) when there are enough
-// of them.  When all blocks are resident anyway, or shared memory lets no more in, the registers
-// of fewer (FEW) serve a block better.  One output, tanh (72 and 96 registers): 1024 wide at 5,000
-// points, loss 94 and 67 us, gradient 211 and 182; 256 wide at 60,000 points, gradient 202 and 262.
-// Three outputs, sine (128 and 168): 256 wide at 5,000 points, 71 and 66; BF16 at 60,000, 217 and 263.
+// blocks beside it hide that latency: as many per SM as registers allow (MANY) when that saves a
+// round of blocks.  Where it does not (all blocks are resident anyway, shared memory lets no more in,
+// or the last round is as empty), the registers of fewer (FEW) serve a block better.  One output,
+// tanh (72 and 96 registers): 1024 wide at 5,000 points, loss 94 and 67 us, gradient 211 and 182; 256
+// wide at 60,000 points, gradient 202 and 262.  Three outputs, sine (128 and 168): 256 wide at
+// 5,000 points, 71 and 66; BF16 at 60,000, 217 and 263; 128 wide at 50,000, 169 and 140.
 template <typename T, int D, bool FAST, bool SINE>
 cudaError_t out_loss_launch(pinn_handle* h, const OutArgs& a, int nblocks, size_t smem, cudaStream_t st) {
   if (a.segpart) return out_loss_blocks_launch<T, D, FAST, SINE, true, D == 1 ? 5 : 4>(h, a, nblocks, smem, st);
-  constexpr int FEW = SINE ? 3 : D == 1 ? 5 : 4, MANY = SINE ? (D == 1 ? 3 : 4) : D == 1 ? 7 : 4;
+  constexpr int FEW = (SINE || D == 3) ? 3 : 5, MANY = D == 3 ? 4 : SINE ? 3 : 7;
   constexpr size_t SM_BYTES = 228 * 1024, BLOCK_EXTRA = 1024 + 64;   // what the system and the static arrays take
-  const bool few = nblocks <= FEW * (int64_t)h->sm_count || SM_BYTES / (smem + BLOCK_EXTRA) < (size_t)MANY;
+  const int sms = std::max(h->sm_count, 1);
+  auto rounds = [&](int per_sm) { return (nblocks + (int64_t)per_sm * sms - 1) / ((int64_t)per_sm * sms); };
+  const bool few = rounds(FEW) <= rounds(MANY) || SM_BYTES / (smem + BLOCK_EXTRA) < (size_t)MANY;
   return few ? out_loss_blocks_launch<T, D, FAST, SINE, false, FEW>(h, a, nblocks, smem, st)
              : out_loss_blocks_launch<T, D, FAST, SINE, false, MANY>(h, a, nblocks, smem, st);
 }

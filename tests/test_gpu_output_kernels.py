@@ -75,6 +75,7 @@ def test_register_output_kernel_other_widths(cuda_lib, widths):
 @pytest.mark.parametrize("pde,activation,n_res", [
     ("burgers", "tanh", 48500), ("burgers", "tanh", 48700),   # 760 blocks: the line between the two register limits
     ("ns", "sine", 29100), ("ns", "sine", 29200),             # 456 blocks
+    ("ns", "tanh", 38800), ("ns", "tanh", 39000),             # 608 blocks: two rounds either way from here on
     ("ns", "tanh", 200), ("burgers", "sine", 200),
 ])
 def test_output_kernel_register_limits(cuda_lib, pde, activation, n_res):
