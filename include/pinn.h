@@ -399,8 +399,9 @@ PINN_API pinn_status pinn_debug_wait_expiry(pinn_handle* h, int M, int N, int K,
  * (up to 2,000,000), the tcgen05 kernels of every pass of h (loss, gradient; single and
  * paired CTAs, the one-kernel forward, the fused adjoint) are launched with an arrival that never
  * comes: their MMA-issuing thread first waits on an mbarrier of its own, or its operands are not
- * brought.  Every wait of these kernels is bounded by wait_us microseconds.  They end as in pinn_debug_wait_expiry; the pass's results are
- * undefined and pinn_status_poll(h) reports PINN_ERR_TIMEOUT.  0 switches it off. */
+ * brought.  Every wait of these kernels is bounded by wait_us microseconds.  They end as in
+ * pinn_debug_wait_expiry; the pass's results are undefined and pinn_status_poll(h) reports
+ * PINN_ERR_TIMEOUT.  0 switches it off. */
 PINN_API pinn_status pinn_debug_stall(pinn_handle* h, int64_t wait_us);
 
 /* ---- many independent networks in one training step --------------------------------
