@@ -31,7 +31,9 @@ class SmemLimits {
     if (e != ok) return e;
     std::lock_guard<std::mutex> lock(add_);
     const int n = n_.load(std::memory_order_relaxed);
-    if (n < MAX) {   // (beyond that every call asks)
+    bool known = false;   // (another thread was faster)
+    for (int i = 0; i < n; ++i) known = known || kern_[i] == kern;
+    if (!known && n < MAX) {   // (beyond that every call asks)
       kern_[n] = kern;
       limit_[n] = limit;
       n_.store(n + 1, std::memory_order_release);
